@@ -738,6 +738,7 @@ struct BatchPlan {
     uint64_t olt_need = 0, leaf_need = 0, rst_need = 0, fill_need = 0;
     uint64_t level_cap[ASK_MAX_LEVELS] = {};  // bound on each level's regions over the frames
     uint32_t total0 = 0;
+    uint32_t leaf_side = 0;               // largest nominal leaf side over the frames
     // the persistent batch kernel: queue items (every level's chunk items and
     // fill bands of every frame), chunk states, level-0 items and states
     uint64_t q_items = 0, q_states = 0, q_total0 = 0, q_states0 = 0;
@@ -815,6 +816,7 @@ ask_status plan_batch(ask_ctx *ctx, const ask_frame *frames, uint32_t nframes, u
         if (d.chunks[0] > 1u)
             bp.q_states0 += regions0;
         bp.leaf_need += plan.max_regions[plan.levels - 1];
+        bp.leaf_side = std::max(bp.leaf_side, plan.side[plan.levels - 1]);
         total0 += (uint64_t)plan.axis0 * plan.axis0;
         if (plan.levels > bp.L)
             bp.L = plan.levels;
@@ -938,6 +940,7 @@ ask_status enqueue_batch(ask_ctx *ctx, const BatchBuffers &b, const BatchPlan &b
     la.fill_cap = bp.fill_need ? (uint32_t)b.fill_cap : 0u;
     la.leaves = b.leaves;
     la.leaf_cap = (uint32_t)b.leaf_cap;
+    la.side = bp.leaf_side;
     la.skip_perimeter = exact ? 1u : 0u;
     la.frames = b.frames;
     la.ctr = b.ctr;

@@ -191,8 +191,8 @@ struct LeafArgs {
     uint32_t n;
     PixelMap pm;
     uint32_t max_dwell;
-    uint32_t side;        // nominal side of the leaf regions
     // both
+    uint32_t side;        // nominal side of the leaf regions (a batch: the largest)
     const void *leaves;   // uint2 (single frame) or uint4 (batch) records
     uint32_t leaf_cap;    // capacity of the leaf list
     uint32_t skip_perimeter;  // leaf perimeters are already in the map

@@ -629,6 +629,7 @@ __global__ void __launch_bounds__(kRefillWarps * 32, BATCH ? kRefillMinBlocksBat
     src.leaves = static_cast<const typename Rec<BATCH>::T *>(a.leaves);
     src.cap = a.leaf_cap;
     leaf_extent(a.ctr, a.leaf_cap, src.front, src.total);
+    src.shift = leaf_item_shift(src.total, a.side, gridDim.x * (uint32_t)kRefillWarps);
     uint32_t srcst = SRC_MORE;
     LeafCursor lc;
     lc.rem = lc.row0 = lc.col0 = lc.ox = lc.oy = lc.frame = 0;
