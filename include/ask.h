@@ -165,7 +165,8 @@ typedef struct {
     uint64_t fill_pixels;                      /* ASK_FLAG_COUNT only */
     uint64_t leaf_pixels;                      /* ASK_FLAG_COUNT only */
     uint64_t border_pixels;                    /* ASK_FLAG_COUNT only */
-    uint64_t iterations;                       /* ASK_FLAG_COUNT only: z-updates executed */
+    uint64_t iterations;                       /* ASK_FLAG_COUNT only: z-updates counted (an orbit
+                                                * found to repeat itself counts max_dwell) */
     uint64_t iterations_per_level[ASK_MAX_LEVELS]; /* ASK_FLAG_COUNT, ASK: z-updates of level i */
     uint64_t leaf_iterations;                  /* ASK_FLAG_COUNT, ASK: z-updates of the leaf kernel */
     float ms_total;                            /* device time of the render */

@@ -34,6 +34,61 @@ __device__ __forceinline__ void z_update(float &x, float &y, float cr, float ci)
     y = ny;
 }
 
+// Two orbits side by side: one update of each, the same operations and bits
+// as z_update.  The real part stays scalar (its inner operation takes a sign
+// on an operand, which the packed form lacks); the doubling and the imaginary
+// part are packed operations on register pairs.  A packed operation takes the
+// FP32 pipe and the dispatch port twice as long as a scalar one, so the gain is
+// small: a loop of nothing but updates runs 8.0e12 updates/s scalar and
+// 8.3e12 this way (of the pipe's 10.07e12); the leaf kernel at n = 16384 takes
+// 1.09 ms scalar, 0.95 with all but the inner operation packed, 0.94 this way.
+using f32x2 = unsigned long long;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ void z_update2(f32x2 &x, f32x2 &y, f32x2 cr, f32x2 ci)
+{
+    float x0, x1, y0, y1, c0, c1;
+    unpack2(x, x0, x1);
+    unpack2(y, y0, y1);
+    unpack2(cr, c0, c1);
+    const f32x2 nx = pack2(__fmaf_rn(x0, x0, __fmaf_rn(-y0, y0, c0)),
+                           __fmaf_rn(x1, x1, __fmaf_rn(-y1, y1, c1)));
+    y = fma2(add2(x, x), y, ci);
+    x = nx;
+}
+
 // The escape test of the current state: |z|^2 = fma(zr, zr, zi*zi) < 4.
 __device__ __forceinline__ bool z_bounded(float x, float y)
 {

@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(1024) leaf_kernel(LeafArgs a, uint32_t leaf_ca
 // hold two thirds of the updates).  A warp that owned 32 fixed pixels would
 // idle most lanes while one orbit runs on, so each warp takes leaves from a
 // device counter and works in two stages:
-//  * pre-pass: 32 fresh pixels at a time, one per lane, all lanes in
+//  * pre-pass: 64 fresh pixels at a time, two per lane, all lanes in
 //    lockstep, run their first kPrePass updates in unchecked blocks of
 //    kPreBlock with one test per block (see dwell()).  An orbit that escapes
 //    there is resolved on the spot by a binary search over its last block
@@ -587,10 +587,12 @@ __global__ void __launch_bounds__(1024) leaf_kernel(LeafArgs a, uint32_t leaf_ca
 //    per-pixel bookkeeping beyond the lane they run on;
 //  * refill loop over the survivors: each lane carries two orbits; every
 //    round each orbit runs one unchecked block of kLeafUnroll updates; an
-//    orbit that escaped (or has less than a block left) parks its saved
-//    state in the warp's park buffer and its slot takes the next survivor
-//    from the ring at once (the pre-pass tops the ring up when it runs
-//    short);
+//    orbit that escaped (or has less than a block left) waits at the block's
+//    start until kRefillSlots slots wait or are idle; then the waiting ones
+//    go to the warp's park buffer and the free slots take the next survivors
+//    from the ring (the pre-pass tops the ring up when it runs short).  An
+//    orbit that reaches max_dwell at a block's end, or repeats an earlier
+//    state, is written there and then;
 //  * when 32 orbits are parked, the warp finishes them together, one per
 //    lane: a binary search over the parked block finds the exact escape (the
 //    block's midpoint state is parked too, so the first halving costs one
@@ -601,77 +603,79 @@ __global__ void __launch_bounds__(1024) leaf_kernel(LeafArgs a, uint32_t leaf_ca
 //    long orbits), so the warps end on short orbits; once the list has run
 //    out and a warp's orbits fit in one slot per lane, slot 1 folds into
 //    slot 0 and the last rounds update one orbit per lane.
+//
+// What bounds it is issue slots (a packed update pair holds the dispatch port
+// as long as two scalar updates): at n = 16384 (g=16 r=4 B=16) it issues or
+// dispatches on about 92% of its active cycles and the FP32 pipe is busy on
+// 64%.  So what it saves is instructions around the updates.  One pixel a lane
+// in the pre-pass, parking and refilling every round, and the cursor and the
+// limits in registers (48 a thread, spilled) took 1.17-1.20 ms, this form
+// 0.93-0.94 (0.97 without the test for a repeated state); n = 65536 (g=32 r=2
+// B=16) 7.5 -> 6.0 ms; 64 mixed frames in a batch 33.5 -> 29.6 ms.
 // ---------------------------------------------------------------------------
 // The leaf kernel over the leaf list of a launch chain.  Each lane of the
 // refill loop carries two independent orbits, so one round's bookkeeping
 // (votes, refills, parking) serves two blocks of updates, and the two update
 // chains interleave.  Parked orbits and ring entries remember their frame.
 template <bool COUNT, bool BATCH>
-__global__ void __launch_bounds__(kRefillWarps * 32, BATCH ? kRefillMinBlocksBatch : kRefillMinBlocks)
-    leaf_refill_kernel(LeafArgs a)
+__global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocks) leaf_refill_kernel(LeafArgs a)
 {
-    __shared__ float4 park_s[kRefillWarps][kParkCap];  // saved state at the block's start and midpoint
-    __shared__ uint4 park_u[kRefillWarps][kParkCap];   // count, pixel, frame
-    __shared__ float4 ring_s[kRefillWarps][kRingCap];  // survivor state and c
-    __shared__ uint4 ring_u[kRefillWarps][kRingCap];   // count, pixel, frame, block limit
+    __shared__ WarpLeaf<BATCH> shared[kRefillWarps];
+    __shared__ uint3 extent;                           // front, leaves, item shift (LeafList)
     const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        uint32_t front, total;
+        leaf_extent(a.ctr, a.leaf_cap, front, total);
+        extent = make_uint3(front, total,
+                            leaf_item_shift(total, a.side, gridDim.x * (uint32_t)kRefillWarps));
+    }
+    __syncthreads();
     if (a.fills != nullptr && wib == kRefillWarps - 1u)
         drain_fills<BATCH>(a, lane);  // the CTA's fill warp
-    const unsigned lt_mask = (1u << lane) - 1u;
-    float4 *qs = park_s[wib];
-    uint4 *qu = park_u[wib];
-    float4 *rs = ring_s[wib];
-    uint4 *ru = ring_u[wib];
-    uint32_t parked = 0;             // warp-uniform
-    uint32_t ring_h = 0, ring_n = 0;  // warp-uniform: first entry, entries
+    WarpLeaf<BATCH> &w = shared[wib];
+    WarpFill f;
+    f.parked = f.ring_h = f.ring_n = 0;
 
     LeafList<BATCH> src;
     src.leaves = static_cast<const typename Rec<BATCH>::T *>(a.leaves);
     src.cap = a.leaf_cap;
-    leaf_extent(a.ctr, a.leaf_cap, src.front, src.total);
-    src.shift = leaf_item_shift(src.total, a.side, gridDim.x * (uint32_t)kRefillWarps);
+    src.extent = &extent;
     uint32_t srcst = SRC_MORE;
-    LeafCursor lc;
-    lc.rem = lc.row0 = lc.col0 = lc.ox = lc.oy = lc.frame = 0;
-    lc.cw = 1;
-    lc.inv_cw = 1.0f;
-    Slot s0, s1;
-    s0.busy = s1.busy = false;
-    s0.x = s0.y = s0.cr = s0.ci = s1.x = s1.y = s1.cr = s1.ci = 0.0f;
-    s0.d = s1.d = s0.pix = s1.pix = 0;
-    s0.lim = s1.lim = 0;
-    uint32_t f0 = 0, f1 = 0;  // frames of the slots' orbits
+    cursor_reset(w.cursor, lane);
+    Slot s[kSlots];
+#pragma unroll
+    for (int i = 0; i < kSlots; ++i)
+        slot_reset(s[i]);
     unsigned long long it = 0, lpx = 0;
 
     for (;;) {
         // refill idle slots from the ring, topping it up with pre-passes
         // while it holds fewer survivors than idle slots (at most 32)
-        const unsigned i0 = __ballot_sync(kFull, !s0.busy), i1 = __ballot_sync(kFull, !s1.busy);
-        if (i0 | i1) {
-            const uint32_t want = min((uint32_t)(__popc(i0) + __popc(i1)), 32u);
-            while (ring_n < want && srcst == SRC_MORE)
-                pre_pass<COUNT, BATCH>(a, src, lc, srcst, rs, ru, ring_h, ring_n, lane, lt_mask, it,
-                                       lpx);
-            refill_from_ring(s0, s1, f0, f1, rs, ru, ring_h, ring_n, i0, i1, lane, lt_mask);
+        for (;;) {
+            const uint32_t idle = 32u * kSlots - busy_slots<kSlots>(s);
+            if (idle < kRefillSlots || (srcst != SRC_MORE && f.ring_n == 0))
+                break;
+            const uint32_t want = min(idle, 32u);
+            while (f.ring_n < want && srcst == SRC_MORE)
+                pre_pass<COUNT, BATCH>(a, src, srcst, w, f, lane, it, lpx);
+            refill_from_ring<BATCH, kSlots>(a, w, f, s);
         }
         // once the leaves have run out and the orbits left fit in one slot
         // per lane, the tail runs on slot 0 alone
-        if (srcst != SRC_MORE &&
-            ring_n + (uint32_t)__popc(__ballot_sync(kFull, s0.busy)) +
-                    (uint32_t)__popc(__ballot_sync(kFull, s1.busy)) <= 32u)
+        if (srcst != SRC_MORE && f.ring_n + busy_slots<kSlots>(s) <= 32u)
             break;
-        refill_round<COUNT, BATCH>(a, s0, s1, f0, f1, qs, qu, parked, lane, lt_mask, it, lpx);
+        while (!refill_round<COUNT, BATCH, kSlots>(a, w, f, s, kRefillSlots, lane, it, lpx)) {
+        }
     }
-    fold_slot1(s1, f1, rs, ru, ring_h, ring_n, lt_mask);
-    refill_from_ring(s0, s1, f0, f1, rs, ru, ring_h, ring_n, __ballot_sync(kFull, !s0.busy), 0u, lane,
-                     lt_mask);
-    while (__any_sync(kFull, s0.busy))
-        refill_round<COUNT, BATCH, false>(a, s0, s1, f0, f1, qs, qu, parked, lane, lt_mask, it, lpx);
+    fold_slot1<BATCH>(w, f, s[1]);
+    refill_from_ring<BATCH, 1>(a, w, f, s);
+    while (!refill_round<COUNT, BATCH, 1>(a, w, f, s, 32u, lane, it, lpx)) {
+    }
     if (a.fills != nullptr)
         drain_fills<BATCH>(a, lane);
     // the orbits still parked
-    if (lane < parked) {
-        finish_parked<COUNT, BATCH>(a, qs[lane], qu[lane], it);
+    if (lane < f.parked) {
+        finish_parked<COUNT, BATCH>(a, w.park_s[lane], w.park_u[lane], BATCH ? w.park_f[lane] : 0u, it);
         if (COUNT)
             ++lpx;
     }

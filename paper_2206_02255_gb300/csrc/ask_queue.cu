@@ -50,6 +50,9 @@ namespace {
 
 enum : uint32_t { QITEM_REGION = 0, QITEM_FILL = 1 };
 
+// Resident CTAs per SM: the region items' latency wants more warps than the
+// leaf work alone (64 registers a thread).
+constexpr int kQueueMinBlocks = 4;
 // Leaf rounds between polls of the held region ticket while a warp is busy.
 constexpr uint32_t kQueuePollRounds = 8;
 
@@ -400,19 +403,13 @@ __global__ void queue_init_kernel(QueueArgs q)
 // The persistent kernel: every warp alternates between region items (taken
 // first, as soon as the held ticket's slot is published) and leaf work.
 template <bool COUNT>
-__global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocksBatch) queue_kernel(QueueArgs q, LeafArgs a)
+__global__ void __launch_bounds__(kRefillWarps * 32, kQueueMinBlocks) queue_kernel(QueueArgs q, LeafArgs a)
 {
-    __shared__ float4 park_s[kRefillWarps][kParkCap];
-    __shared__ uint4 park_u[kRefillWarps][kParkCap];
-    __shared__ float4 ring_s[kRefillWarps][kRingCap];
-    __shared__ uint4 ring_u[kRefillWarps][kRingCap];
+    __shared__ WarpLeaf<true> shared[kRefillWarps];
     const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    float4 *qs = park_s[wib];
-    uint4 *qu = park_u[wib];
-    float4 *rs = ring_s[wib];
-    uint4 *ru = ring_u[wib];
-    uint32_t parked = 0, ring_h = 0, ring_n = 0;  // warp-uniform
+    WarpLeaf<true> &w = shared[wib];
+    WarpFill fl;
+    fl.parked = fl.ring_h = fl.ring_n = 0;
 
     uint32_t epoch = 0;
     if (lane == 0)
@@ -424,16 +421,10 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocksBatch) queu
     src.epoch = epoch;
     src.ticket = kNone;
     uint32_t srcst = SRC_MORE;
-    LeafCursor lc;
-    lc.rem = lc.row0 = lc.col0 = lc.ox = lc.oy = lc.frame = 0;
-    lc.cw = 1;
-    lc.inv_cw = 1.0f;
-    Slot s0, s1;
-    s0.busy = s1.busy = false;
-    s0.x = s0.y = s0.cr = s0.ci = s1.x = s1.y = s1.cr = s1.ci = 0.0f;
-    s0.d = s1.d = s0.pix = s1.pix = 0;
-    s0.lim = s1.lim = 0;
-    uint32_t f0 = 0, f1 = 0;
+    cursor_reset(w.cursor, lane);
+    Slot s[2];
+    slot_reset(s[0]);
+    slot_reset(s[1]);
     unsigned long long it = 0, lpx = 0;
 
     uint32_t rt = kNone;      // region ticket held
@@ -478,17 +469,16 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocksBatch) queu
         if (srcst == SRC_WAIT)
             srcst = SRC_MORE;  // ask again
         bool worked = false;
-        const unsigned i0 = __ballot_sync(kFull, !s0.busy), i1 = __ballot_sync(kFull, !s1.busy);
-        if (i0 | i1) {
-            const uint32_t want = min((uint32_t)(__popc(i0) + __popc(i1)), 32u);
-            while (ring_n < want && srcst == SRC_MORE)
-                if (pre_pass<COUNT, true>(a, src, lc, srcst, rs, ru, ring_h, ring_n, lane, lt_mask, it,
-                                          lpx))
+        const uint32_t idle_slots = 64u - busy_slots<2>(s);
+        if (idle_slots) {
+            const uint32_t want = min(idle_slots, 32u);
+            while (fl.ring_n < want && srcst == SRC_MORE)
+                if (pre_pass<COUNT, true>(a, src, srcst, w, fl, lane, it, lpx))
                     worked = true;
-            refill_from_ring(s0, s1, f0, f1, rs, ru, ring_h, ring_n, i0, i1, lane, lt_mask);
+            refill_from_ring<true, 2>(a, w, fl, s);
         }
-        if (__any_sync(kFull, s0.busy || s1.busy)) {
-            refill_round<COUNT, true>(a, s0, s1, f0, f1, qs, qu, parked, lane, lt_mask, it, lpx);
+        if (__any_sync(kFull, s[0].busy || s[1].busy)) {
+            refill_round<COUNT, true, 2>(a, w, fl, s, 1u, lane, it, lpx);
             worked = true;
             ++rounds;
         }
@@ -497,7 +487,7 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocksBatch) queu
             polls = 0;
             continue;
         }
-        if (rclosed && srcst == SRC_DONE && ring_n == 0)
+        if (rclosed && srcst == SRC_DONE && fl.ring_n == 0)
             break;
         // nothing to do now: back off; the count starts again whenever the
         // queue or the leaf list moves
@@ -521,8 +511,8 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocksBatch) queu
         __nanosleep(polls < 32u ? 32u : 256u);
     }
     // the orbits still parked
-    if (lane < parked) {
-        finish_parked<COUNT, true>(a, qs[lane], qu[lane], it);
+    if (lane < fl.parked) {
+        finish_parked<COUNT, true>(a, w.park_s[lane], w.park_u[lane], w.park_f[lane], it);
         if (COUNT)
             ++lpx;
     }

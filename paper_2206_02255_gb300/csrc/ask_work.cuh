@@ -194,15 +194,20 @@ __device__ __forceinline__ void chunk_query(const FView &a, const Region &g, uin
 // Leaf machinery (see the leaf kernel in ask_kernels.cu)
 // ---------------------------------------------------------------------------
 constexpr int kRefillWarps = 8;    // warps per CTA
-// Resident CTAs per SM: the park buffer and the ring take 5 KB of shared
-// memory a warp, so 5 CTAs of 8 warps fit an SM (200 KB) with up to 48
-// registers a thread (one frame); a batch's per-frame lookups need more
-// registers, 4 CTAs.
-constexpr int kRefillMinBlocks = 5;
-constexpr int kRefillMinBlocksBatch = 4;
-constexpr uint32_t kParkCap = 96;  // parked orbits per warp (< 32 + 2 * 32)
-constexpr uint32_t kRingCap = 64;  // survivors per warp (< 32 + 32: topped up while below 32)
+// Resident CTAs per SM.  With two orbits a lane the FP32 pipe is busy enough
+// at 24 warps, and 80 registers leave nothing to spill: at n = 16384 (g=16 r=4
+// B=16) the leaf kernel takes 1.08 ms at 5 CTAs (48 registers, 60 bytes
+// spilled), 0.96 at 4 and 0.93 at 3.
+constexpr int kRefillMinBlocks = 3;
+constexpr int kSlots = 2;          // orbits per lane in the refill loop (four: 0.94-0.99 ms)
+constexpr uint32_t kParkCap = 96;  // parked orbits per warp (fewer than 32 wait, a round adds 64)
+constexpr uint32_t kRingCap = 96;  // survivors per warp (< 32 + 64: topped up while below 32)
+constexpr uint32_t kRawCount = 0xffffffffu;  // count of an orbit that may not run in blocks
 constexpr int kLeafUnroll = 64;    // updates per unchecked block of the refill loop (a power of two)
+// Idle or waiting slots (of 64) before a warp parks and refills: that code
+// costs about a third of a round, and most rounds end a few orbits.  At
+// n = 16384 the leaf kernel took 1.097 ms with 1, 1.077 with 8, 1.095 with 16.
+constexpr uint32_t kRefillSlots = 8;
 constexpr int kPreBlock = 8;       // updates per unchecked block of the pre-pass (a power of two)
 constexpr int kPrePass = 64;       // updates of the pre-pass (a multiple of kPreBlock)
 
@@ -235,18 +240,19 @@ __device__ __forceinline__ LView leaf_view(const LeafArgs &a, uint32_t frame)
 // Exact dwell of a parked orbit: s.xy = state after d updates, known to
 // pass the test, s.zw = the state kLeafUnroll / 2 updates later (the block's
 // midpoint), and "escaped, or d >= max_dwell" known to hold kLeafUnroll
-// updates later.  Points where escape is not absorbing take the tested loop
-// instead.  u = (count, py << 16 | px, frame).
+// updates later.  Points where escape is not absorbing (count kRawCount, at
+// z = 0) take the tested loop instead.  u = (count, py << 16 | px).
 template <bool COUNT, bool BATCH>
-__device__ __forceinline__ void finish_parked(const LeafArgs &a, float4 s, uint4 u,
+__device__ __forceinline__ void finish_parked(const LeafArgs &a, float4 s, uint2 u, uint32_t frame,
                                               unsigned long long &it)
 {
-    const LView v = leaf_view<BATCH>(a, u.z);
+    const LView v = leaf_view<BATCH>(a, frame);
     const uint32_t px = u.y & 0xffffu, py = u.y >> 16;
     const float2 c = pixel_c(v.pm, px, py);
     uint32_t d = u.x;
     float x = s.x, y = s.y;
-    if (!escape_absorbing(c.x, c.y)) {
+    if (d == kRawCount) {
+        d = 0;
         while (d < v.max_dwell && z_bounded(x, y)) {
             z_update(x, y, c.x, c.y);
             ++d;
@@ -326,16 +332,74 @@ __device__ __forceinline__ uint32_t rows_in(uint32_t q, float inv_w)
 // One orbit slot of a lane in the refill loop.
 struct Slot {
     float x, y, cr, ci;
-    uint32_t d, pix;  // count, pixel (py << 16 | px)
-    uint32_t lim;     // a whole unchecked block may run while d < lim
+    float bx, by;     // an earlier state of the orbit (see settle_slot)
+    uint32_t d, pix;  // count (kRawCount: not to run in blocks), pixel (py << 16 | px)
+    uint32_t frame;   // batch: the orbit's frame
+    uint32_t lim;     // batch: slot_limit of its frame
     bool busy;
 };
 
-// The warp's current leaf, handed out as a row-major cursor.
+__device__ __forceinline__ void slot_reset(Slot &s)
+{
+    s.x = s.y = s.cr = s.ci = s.bx = s.by = 0.0f;
+    s.d = s.pix = s.frame = s.lim = 0;
+    s.busy = false;
+}
+
+// A whole unchecked block may run while d < limit: kLeafUnroll - 1 below
+// max_dwell, 0 if no block fits.
+__device__ __forceinline__ uint32_t block_limit(uint32_t max_dwell)
+{
+    return max_dwell >= (uint32_t)kLeafUnroll ? max_dwell - (uint32_t)kLeafUnroll + 1u : 0u;
+}
+
+template <bool BATCH>
+__device__ __forceinline__ uint32_t slot_limit(const LeafArgs &a, const Slot &s)
+{
+    return BATCH ? s.lim : block_limit(a.max_dwell);
+}
+
+// The warp's current leaf, handed out as a row-major cursor.  It lives in
+// shared memory between pre-passes, out of the refill loop's registers.
 struct LeafCursor {
     uint32_t rem, row0, col0, ox, oy, cw, frame;
     float inv_cw;
 };
+
+// An empty cursor (lane 0 writes, the warp sees it).
+__device__ __forceinline__ void cursor_reset(LeafCursor &lc, uint32_t lane)
+{
+    if (lane == 0) {
+        lc.rem = lc.row0 = lc.col0 = lc.ox = lc.oy = lc.frame = 0;
+        lc.cw = 1;
+        lc.inv_cw = 1.0f;
+    }
+    __syncwarp();
+}
+
+// A warp's share of the leaf kernel's shared memory: parked orbits (the
+// states at their block's start and midpoint; count and pixel), the ring of
+// survivors (state, pixel, count) and the leaf cursor.
+template <bool BATCH>
+struct WarpLeaf {
+    float4 park_s[kParkCap];
+    float4 ring[kRingCap];
+    uint2 park_u[kParkCap];
+    uint32_t park_f[BATCH ? kParkCap : 1], ring_f[BATCH ? kRingCap : 1];  // frames
+    LeafCursor cursor;
+};
+
+// Warp-uniform fill levels: parked orbits, the ring's first entry and entries.
+struct WarpFill {
+    uint32_t parked, ring_h, ring_n;
+};
+
+__device__ __forceinline__ unsigned lanes_below()
+{
+    unsigned m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
 
 // Where the pre-pass takes its leaves from.
 enum : uint32_t {
@@ -412,8 +476,9 @@ __device__ __forceinline__ uint32_t leaf_item_shift(uint32_t leaves, uint32_t si
 template <bool BATCH>
 struct LeafList {
     const typename Rec<BATCH>::T *leaves;
-    uint32_t front, total, cap;
-    uint32_t shift;  // an item is one of 1 << shift row bands of a leaf
+    uint32_t cap;
+    const uint3 *extent;  // in shared memory: entries of the front, entries,
+                          // shift (an item is one of 1 << shift bands of a leaf)
 
     __device__ __forceinline__ uint32_t next(const LeafArgs &a, LeafCursor &lc, uint32_t lane)
     {
@@ -422,10 +487,10 @@ struct LeafList {
         if (lane == 0)
             li = atomicAdd(&a.ctr->leaf_work, 1u);
         li = __shfl_sync(kFull, li, 0);
-        const uint32_t leaf = li >> shift;
-        if (leaf >= total)
+        const uint32_t shift = extent->z, leaf = li >> shift;
+        if (leaf >= extent->y)
             return SRC_DONE;
-        const typename R::T e = leaves[table_slot(leaf, front, cap)];
+        const typename R::T e = leaves[table_slot(leaf, extent->x, cap)];
         const Region g = R::region(e);
         const bool skip = a.skip_perimeter != 0u;
         if (shift) {
@@ -450,38 +515,56 @@ struct LeafList {
     }
 };
 
-// Pre-pass: up to 32 fresh pixels from the leaf cursor, the j-th on lane j,
-// run their first kPrePass updates in lockstep (unchecked blocks of
-// kPreBlock, one test each, only while a whole block stays within
-// max_dwell).  An orbit whose block ends escaped has its dwell in that block:
-// a binary search over the block (kPreBlock - 1 updates and log2(kPreBlock)
-// tests, the same on every lane) finds it, and the dwell is written.  Every
-// other pixel is pushed onto the ring with its state: survivors of the whole
-// pass, orbits stopped by max_dwell, and points where escape is not
-// absorbing (d = 0; the refill loop parks them at once and finish_parked
-// runs the tested loop).  Leaves come from `src` (see LeafList); `srcst`
-// becomes SRC_WAIT or SRC_DONE when it has none to give.  Returns the number
-// of pixels taken.
+// Put a survivor on the ring, `rank` entries past its end.
+template <bool BATCH>
+__device__ __forceinline__ void push_survivor(WarpLeaf<BATCH> &w, const WarpFill &f, uint32_t rank,
+                                              float x, float y, uint32_t pix, uint32_t d, uint32_t frame)
+{
+    uint32_t k = f.ring_h + f.ring_n + rank;
+    if (k >= kRingCap)
+        k -= kRingCap;
+    w.ring[k] = make_float4(x, y, __uint_as_float(pix), __uint_as_float(d));
+    if (BATCH)
+        w.ring_f[k] = frame;
+}
+
+// Pre-pass: up to 64 fresh pixels from the leaf cursor, the j-th on lane
+// j & 31 (two a lane, side by side), run their first kPrePass updates in
+// lockstep: unchecked blocks of kPreBlock, one test each, only while a whole
+// block stays within max_dwell.  A pixel whose block fails the test goes back
+// to the block's start and repeats it (with the same end) until every pixel
+// has failed or the pass is over.  A failed block holds the pixel's dwell: a
+// binary search over it (kPreBlock - 1 updates and log2(kPreBlock) tests, the
+// same on every lane) finds it, and the dwell is written.  Every other pixel
+// is pushed onto the ring with its state: survivors of the whole pass, orbits
+// stopped by max_dwell, and points where escape is not absorbing (kRawCount;
+// the refill loop parks them and finish_parked runs the tested loop).  Leaves
+// come from `src` (see LeafList); `srcst` becomes SRC_WAIT or SRC_DONE when it
+// has none to give.  Returns the number of pixels taken.
 template <bool COUNT, bool BATCH, typename Src>
-__device__ __forceinline__ uint32_t pre_pass(const LeafArgs &a, Src &src, LeafCursor &lc,
-                                             uint32_t &srcst, float4 *rs, uint4 *ru, uint32_t ring_h,
-                                             uint32_t &ring_n, uint32_t lane, unsigned lt_mask,
+__device__ __forceinline__ uint32_t pre_pass(const LeafArgs &a, Src &src, uint32_t &srcst,
+                                             WarpLeaf<BATCH> &w, WarpFill &f, uint32_t lane,
                                              unsigned long long &it, unsigned long long &lpx)
 {
-    uint32_t pix = 0, frame = 0;
-    bool have = false;
+    uint32_t pix0 = 0, pix1 = 0, fr0 = 0, fr1 = 0;
     uint32_t base = 0;
-    while (base < 32u && srcst == SRC_MORE) {
+    LeafCursor lc = w.cursor;
+    while (base < 64u && srcst == SRC_MORE) {
         if (lc.rem == 0) {
             srcst = src.next(a, lc, lane);
             continue;
         }
-        const uint32_t take = min(32u - base, lc.rem);
-        if (lane >= base && lane < base + take) {
-            const uint32_t q = lc.col0 + (lane - base), dr = rows_in(q, lc.inv_cw);
-            pix = ((lc.oy + lc.row0 + dr) << 16) | (lc.ox + q - dr * lc.cw);
-            frame = lc.frame;
-            have = true;
+        const uint32_t take = min(64u - base, lc.rem);
+        const uint32_t j0 = lane - base, j1 = lane + 32u - base;  // (wrap below base)
+        if (j0 < take) {
+            const uint32_t q = lc.col0 + j0, dr = rows_in(q, lc.inv_cw);
+            pix0 = ((lc.oy + lc.row0 + dr) << 16) | (lc.ox + q - dr * lc.cw);
+            fr0 = lc.frame;
+        }
+        if (j1 < take) {
+            const uint32_t q = lc.col0 + j1, dr = rows_in(q, lc.inv_cw);
+            pix1 = ((lc.oy + lc.row0 + dr) << 16) | (lc.ox + q - dr * lc.cw);
+            fr1 = lc.frame;
         }
         const uint32_t q = lc.col0 + take, dr = rows_in(q, lc.inv_cw);
         lc.col0 = q - dr * lc.cw;
@@ -489,235 +572,301 @@ __device__ __forceinline__ uint32_t pre_pass(const LeafArgs &a, Src &src, LeafCu
         lc.rem -= take;
         base += take;
     }
+    __syncwarp();
+    if (lane == 0)
+        w.cursor = lc;
+    __syncwarp();
     if (base == 0)
         return 0;
-    const LView v = leaf_view<BATCH>(a, frame);
-    const uint32_t px = pix & 0xffffu, py = pix >> 16;
-    const float2 c = pixel_c(v.pm, px, py);
-    const bool absorbing = escape_absorbing(c.x, c.y);
-    // A lane runs while its orbit passes every block's test; (ex, ey) keeps
-    // the state a stopped lane stopped at (the start of its escaping block,
-    // or, in a batch, the state its own max_dwell left no room beyond), so
-    // a stopped lane's (x, y) may run on to garbage with no rollback.  d
-    // counts only the blocks a lane ran.
-    float x = 0.0f, y = 0.0f, ex = 0.0f, ey = 0.0f;
-    uint32_t d = 0;
-    bool run = have && absorbing, esc = false;
+    const bool have0 = lane < base, have1 = lane + 32u < base;
+    const float2 c0 = pixel_c(leaf_view<BATCH>(a, fr0).pm, pix0 & 0xffffu, pix0 >> 16);
+    const float2 c1 = pixel_c(leaf_view<BATCH>(a, fr1).pm, pix1 & 0xffffu, pix1 >> 16);
+    const uint32_t cap0 = leaf_view<BATCH>(a, fr0).max_dwell, cap1 = leaf_view<BATCH>(a, fr1).max_dwell;
+    const bool go0 = have0 && escape_absorbing(c0.x, c0.y);
+    const bool go1 = have1 && escape_absorbing(c1.x, c1.y);
+    const f32x2 cr = pack2(c0.x, c1.x), ci = pack2(c0.y, c1.y);
+    constexpr uint32_t KP = (uint32_t)kPreBlock;
+    float x0 = 0.0f, y0 = 0.0f, x1 = 0.0f, y1 = 0.0f;
+    uint32_t d0 = 0, d1 = 0;
+    bool run0 = go0, run1 = go1;  // passed every block so far
     // one frame: the blocks that fit below max_dwell, the same for every lane
     const uint32_t nb = BATCH ? (uint32_t)(kPrePass / kPreBlock)
-                              : min((uint32_t)(kPrePass / kPreBlock), v.max_dwell / (uint32_t)kPreBlock);
+                              : min((uint32_t)(kPrePass / kPreBlock), a.max_dwell / KP);
 #pragma unroll
     for (int b = 0; b < kPrePass / kPreBlock; ++b) {
         if (!BATCH && (uint32_t)b >= nb)
             break;
-        if (BATCH) {
-            const bool fits = v.max_dwell - d >= (uint32_t)kPreBlock;  // a whole block fits
-            if (run && !fits) {
-                ex = x;
-                ey = y;
-            }
-            run = run && fits;
-        }
-        if (!__any_sync(kFull, run))
-            break;
-        const float sx = x, sy = y;
+        f32x2 x = pack2(x0, x1), y = pack2(y0, y1);
 #pragma unroll
         for (int k = 0; k < kPreBlock; ++k)
-            z_update(x, y, c.x, c.y);
-        const bool ok = z_bounded(x, y);
-        if (run && !ok) {
-            esc = true;  // the dwell lies in (d, d + kPreBlock]
-            ex = sx;
-            ey = sy;
-        }
-        if (run && ok)
-            d += (uint32_t)kPreBlock;
-        run = run && ok;
+            z_update2(x, y, cr, ci);
+        float m0, m1, e0, e1;
+        unpack2(fma2(x, x, mul2(y, y)), m0, m1);
+        run0 = go0 && m0 < 4.0f && (!BATCH || cap0 - d0 >= KP);
+        run1 = go1 && m1 < 4.0f && (!BATCH || cap1 - d1 >= KP);
+        unpack2(x, e0, e1);
+        x0 = run0 ? e0 : x0;
+        x1 = run1 ? e1 : x1;
+        unpack2(y, e0, e1);
+        y0 = run0 ? e0 : y0;
+        y1 = run1 ? e1 : y1;
+        d0 += run0 ? KP : 0u;
+        d1 += run1 ? KP : 0u;
+        if (!__any_sync(kFull, run0 || run1))
+            break;
     }
-    if (run) {
-        ex = x;
-        ey = y;
-    }
-    if (__any_sync(kFull, esc)) {
-        // invariant: the state at count d passes the test and the state at
-        // d + 2h fails; halve h until the first failing count is d + 1
-        float rx = ex, ry = ey;
-        uint32_t rd = d;
+    const bool esc0 = go0 && !run0 && (!BATCH || cap0 - d0 >= KP);
+    const bool esc1 = go1 && !run1 && (!BATCH || cap1 - d1 >= KP);
+    if (__any_sync(kFull, esc0 || esc1)) {
+        // invariant: the state at count r passes the test and the state at
+        // r + 2h fails; halve h until the first failing count is r + 1
+        float rx0 = x0, ry0 = y0, rx1 = x1, ry1 = y1;
+        uint32_t r0 = d0, r1 = d1;
 #pragma unroll
-        for (uint32_t h = (uint32_t)kPreBlock / 2u; h >= 1u; h >>= 1) {
-            float tx = rx, ty = ry;
+        for (uint32_t h = KP / 2u; h >= 1u; h >>= 1) {
+            f32x2 x = pack2(rx0, rx1), y = pack2(ry0, ry1);
 #pragma unroll
             for (uint32_t k = 0; k < h; ++k)
-                z_update(tx, ty, c.x, c.y);
-            if (z_bounded(tx, ty)) {
-                rx = tx;
-                ry = ty;
-                rd += h;
+                z_update2(x, y, cr, ci);
+            float m0, m1, e0, e1;
+            unpack2(fma2(x, x, mul2(y, y)), m0, m1);
+            unpack2(x, e0, e1);
+            rx0 = m0 < 4.0f ? e0 : rx0;
+            rx1 = m1 < 4.0f ? e1 : rx1;
+            unpack2(y, e0, e1);
+            ry0 = m0 < 4.0f ? e0 : ry0;
+            ry1 = m1 < 4.0f ? e1 : ry1;
+            r0 += m0 < 4.0f ? h : 0u;
+            r1 += m1 < 4.0f ? h : 0u;
+        }
+        if (esc0) {
+            const LView v = leaf_view<BATCH>(a, fr0);
+            v.map[(size_t)(pix0 >> 16) * v.n + (pix0 & 0xffffu)] = r0 + 1u;
+            if (COUNT) {
+                it += r0 + 1u;
+                ++lpx;
             }
         }
-        if (esc) {
-            v.map[(size_t)py * v.n + px] = rd + 1u;
+        if (esc1) {
+            const LView v = leaf_view<BATCH>(a, fr1);
+            v.map[(size_t)(pix1 >> 16) * v.n + (pix1 & 0xffffu)] = r1 + 1u;
             if (COUNT) {
-                it += rd + 1u;
+                it += r1 + 1u;
                 ++lpx;
             }
         }
     }
-    const bool push = have && !esc;
-    const unsigned pm = __ballot_sync(kFull, push);
-    if (push) {
-        uint32_t slot = ring_h + ring_n + (uint32_t)__popc(pm & lt_mask);
-        if (slot >= kRingCap)
-            slot -= kRingCap;
-        const uint32_t K = (uint32_t)kLeafUnroll;
-        const uint32_t lim = (absorbing && v.max_dwell >= K) ? v.max_dwell - K + 1u : 0u;
-        rs[slot] = make_float4(ex, ey, c.x, c.y);
-        ru[slot] = make_uint4(d, pix, frame, lim);
-    }
-    ring_n += (uint32_t)__popc(pm);
+    const bool push0 = have0 && !esc0, push1 = have1 && !esc1;
+    const unsigned p0 = __ballot_sync(kFull, push0), p1 = __ballot_sync(kFull, push1);
+    const unsigned lt = lanes_below();
+    if (push0)
+        push_survivor<BATCH>(w, f, (uint32_t)__popc(p0 & lt), x0, y0, pix0, go0 ? d0 : kRawCount, fr0);
+    if (push1)
+        push_survivor<BATCH>(w, f, (uint32_t)(__popc(p0) + __popc(p1 & lt)), x1, y1, pix1,
+                             go1 ? d1 : kRawCount, fr1);
+    f.ring_n += (uint32_t)(__popc(p0) + __popc(p1));
     __syncwarp();
     return base;
 }
 
+// Take ring entry `rank` from the front into an idle slot.
+template <bool BATCH>
+__device__ __forceinline__ void take_survivor(const LeafArgs &a, const WarpLeaf<BATCH> &w,
+                                              const WarpFill &f, uint32_t rank, Slot &s)
+{
+    uint32_t k = f.ring_h + rank;
+    if (k >= kRingCap)
+        k -= kRingCap;
+    const float4 e = w.ring[k];
+    s.frame = BATCH ? w.ring_f[k] : 0u;
+    s.pix = __float_as_uint(e.z);
+    s.d = __float_as_uint(e.w);
+    const LView v = leaf_view<BATCH>(a, s.frame);
+    const float2 c = pixel_c(v.pm, s.pix & 0xffffu, s.pix >> 16);
+    s.x = s.bx = e.x;
+    s.y = s.by = e.y;
+    s.cr = c.x;
+    s.ci = c.y;
+    if (BATCH)
+        s.lim = block_limit(v.max_dwell);
+    s.busy = true;
+}
 
 // Refill the idle slots of the refill loop from the ring of survivors: slot 0
-// of the idle lanes first, then slot 1 (i0, i1: ballots of the idle slots).
-__device__ __forceinline__ void refill_from_ring(Slot &s0, Slot &s1, uint32_t &f0, uint32_t &f1,
-                                                 const float4 *rs, const uint4 *ru, uint32_t &ring_h,
-                                                 uint32_t &ring_n, unsigned i0, unsigned i1,
-                                                 uint32_t lane, unsigned lt_mask)
+// of the idle lanes first, then slot 1, ...  Returns the orbits taken.
+template <bool BATCH, int NS>
+__device__ __forceinline__ uint32_t refill_from_ring(const LeafArgs &a, const WarpLeaf<BATCH> &w,
+                                                     WarpFill &f, Slot *s)
 {
-    const uint32_t n0 = (uint32_t)__popc(i0);
-    const uint32_t take = min(n0 + (uint32_t)__popc(i1), ring_n);
-    const uint32_t r0 = (uint32_t)__popc(i0 & lt_mask);
-    const uint32_t r1 = n0 + (uint32_t)__popc(i1 & lt_mask);
-    if (!s0.busy && r0 < take) {
-        uint32_t k = ring_h + r0;
-        if (k >= kRingCap)
-            k -= kRingCap;
-        const float4 sv = rs[k];
-        const uint4 uv = ru[k];
-        s0.x = sv.x;
-        s0.y = sv.y;
-        s0.cr = sv.z;
-        s0.ci = sv.w;
-        s0.d = uv.x;
-        s0.pix = uv.y;
-        f0 = uv.z;
-        s0.lim = uv.w;
-        s0.busy = true;
+    const unsigned lt = lanes_below();
+    uint32_t n = 0;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        const unsigned idle = __ballot_sync(kFull, !s[i].busy);
+        const uint32_t r = n + (uint32_t)__popc(idle & lt);
+        if (!s[i].busy && r < f.ring_n)
+            take_survivor<BATCH>(a, w, f, r, s[i]);
+        n += (uint32_t)__popc(idle);
     }
-    if (!s1.busy && r1 < take) {
-        uint32_t k = ring_h + r1;
-        if (k >= kRingCap)
-            k -= kRingCap;
-        const float4 sv = rs[k];
-        const uint4 uv = ru[k];
-        s1.x = sv.x;
-        s1.y = sv.y;
-        s1.cr = sv.z;
-        s1.ci = sv.w;
-        s1.d = uv.x;
-        s1.pix = uv.y;
-        f1 = uv.z;
-        s1.lim = uv.w;
-        s1.busy = true;
-    }
-    ring_h += take;
-    if (ring_h >= kRingCap)
-        ring_h -= kRingCap;
-    ring_n -= take;
+    n = min(n, f.ring_n);
+    f.ring_h += n;
+    if (f.ring_h >= kRingCap)
+        f.ring_h -= kRingCap;
+    f.ring_n -= n;
     __syncwarp();
+    return n;
+}
+
+// Orbits in the first NS slots of the warp.
+template <int NS>
+__device__ __forceinline__ uint32_t busy_slots(const Slot *s)
+{
+    uint32_t n = 0;
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+        n += (uint32_t)__popc(__ballot_sync(kFull, s[i].busy));
+    return n;
 }
 
 // Move the orbits of slot 1 onto the ring (the ring and both slots hold at
 // most 32 orbits between them when this is called), so the refill that
 // follows puts every orbit in slot 0 and the rounds after it update one
 // orbit per lane: once the leaves have run out and few orbits are left, a
-// round then costs half the instructions.
-__device__ __forceinline__ void fold_slot1(Slot &s1, uint32_t f1, float4 *rs, uint4 *ru,
-                                           uint32_t ring_h, uint32_t &ring_n, unsigned lt_mask)
+// round then costs half the work.
+template <bool BATCH>
+__device__ __forceinline__ void fold_slot1(WarpLeaf<BATCH> &w, WarpFill &f, Slot &s1)
 {
-    const unsigned b1 = __ballot_sync(kFull, s1.busy);
+    const unsigned b = __ballot_sync(kFull, s1.busy);
     if (s1.busy) {
-        uint32_t slot = ring_h + ring_n + (uint32_t)__popc(b1 & lt_mask);
-        if (slot >= kRingCap)
-            slot -= kRingCap;
-        rs[slot] = make_float4(s1.x, s1.y, s1.cr, s1.ci);
-        ru[slot] = make_uint4(s1.d, s1.pix, f1, s1.lim);
+        push_survivor<BATCH>(w, f, (uint32_t)__popc(b & lanes_below()), s1.x, s1.y, s1.pix, s1.d, s1.frame);
         s1.busy = false;
     }
-    ring_n += (uint32_t)__popc(b1);
+    f.ring_n += (uint32_t)__popc(b);
     __syncwarp();
 }
 
-// One round of the refill loop: an unchecked block of kLeafUnroll updates on
-// both slots (TWO) or on slot 0 alone (the results of a slot that is idle or
-// parks are not used); an orbit that escaped in the block, has less than a
-// block left below max_dwell or has |c| near 2 parks its state before the
-// block (and the block's midpoint state) in the park buffer; whenever 32
-// orbits are parked the warp finishes them together.
-template <bool COUNT, bool BATCH, bool TWO = true>
-__device__ __forceinline__ void refill_round(const LeafArgs &a, Slot &s0, Slot &s1, uint32_t f0,
-                                             uint32_t f1, float4 *qs, uint4 *qu, uint32_t &parked,
-                                             uint32_t lane, unsigned lt_mask, unsigned long long &it,
-                                             unsigned long long &lpx)
+// Settle a slot after a block (x, y: the state after it): an orbit
+// that passed the block's test counts it, and is done, at max_dwell, when the
+// block ends there (the block limit lim stands K - 1 below max_dwell) or when
+// its state equals the saved one (bx, by): the iteration is a function of the
+// state alone, so an orbit that repeats a state repeats it for ever and never
+// escapes.  (Equal up to the sign of a zero, which changes no magnitude and
+// no test.)  The saved state is renewed whenever d / K is a power of two, so a
+// cycle is seen within twice the updates it took to enter it, if its length
+// divides a multiple of K below d.  An orbit that failed the test, or has less
+// than a block left, stays at the block's start and waits there to be parked
+// (running the block again changes nothing).  Returns whether it waits.
+template <bool COUNT, bool BATCH>
+__device__ __forceinline__ bool settle_slot(const LeafArgs &a, Slot &s, float x, float y,
+                                            unsigned long long &it, unsigned long long &lpx)
 {
     const uint32_t K = (uint32_t)kLeafUnroll;
-    const float sx0 = s0.x, sy0 = s0.y, sx1 = s1.x, sy1 = s1.y;
-#pragma unroll
-    for (int k = 0; k < kLeafUnroll / 2; ++k) {
-        z_update(s0.x, s0.y, s0.cr, s0.ci);
-        if (TWO)
-            z_update(s1.x, s1.y, s1.cr, s1.ci);
+    const uint32_t lim = slot_limit<BATCH>(a, s);
+    const bool ok = s.d < lim && z_bounded(x, y);
+    if (ok) {
+        s.x = x;
+        s.y = y;
     }
-    const float mx0 = s0.x, my0 = s0.y, mx1 = s1.x, my1 = s1.y;  // midpoint states
-#pragma unroll
-    for (int k = 0; k < kLeafUnroll / 2; ++k) {
-        z_update(s0.x, s0.y, s0.cr, s0.ci);
-        if (TWO)
-            z_update(s1.x, s1.y, s1.cr, s1.ci);
-    }
-    bool park0 = false, park1 = false;
-    if (s0.busy) {
-        if (s0.d < s0.lim && z_bounded(s0.x, s0.y))
-            s0.d += K;
-        else
-            park0 = true;
-    }
-    if (TWO && s1.busy) {
-        if (s1.d < s1.lim && z_bounded(s1.x, s1.y))
-            s1.d += K;
-        else
-            park1 = true;
-    }
-    const unsigned p0 = __ballot_sync(kFull, park0), p1 = __ballot_sync(kFull, park1);
-    if (p0 | p1) {
-        const uint32_t n0 = (uint32_t)__popc(p0);
-        if (park0) {
-            const uint32_t slot = parked + (uint32_t)__popc(p0 & lt_mask);
-            qs[slot] = make_float4(sx0, sy0, mx0, my0);
-            qu[slot] = make_uint4(s0.d, s0.pix, f0, 0u);
-            s0.busy = false;
-        }
-        if (park1) {
-            const uint32_t slot = parked + n0 + (uint32_t)__popc(p1 & lt_mask);
-            qs[slot] = make_float4(sx1, sy1, mx1, my1);
-            qu[slot] = make_uint4(s1.d, s1.pix, f1, 0u);
-            s1.busy = false;
-        }
-        parked += n0 + (uint32_t)__popc(p1);
-        __syncwarp();
-        while (parked >= 32u) {
-            parked -= 32u;
-            const float4 sv = qs[parked + lane];
-            const uint4 uv = qu[parked + lane];
-            __syncwarp();
-            finish_parked<COUNT, BATCH>(a, sv, uv, it);
-            if (COUNT)
+    if (s.busy && ok) {
+        s.d += K;
+        const uint32_t md = lim + K - 1u;
+        if (s.d == md || (x == s.bx && y == s.by)) {
+            const LView v = leaf_view<BATCH>(a, s.frame);
+            v.map[(size_t)(s.pix >> 16) * v.n + (s.pix & 0xffffu)] = md;
+            if (COUNT) {
+                it += md;
                 ++lpx;
+            }
+            s.busy = false;
+        } else if (((s.d / K) & (s.d / K - 1u)) == 0u) {
+            s.bx = x;
+            s.by = y;
         }
     }
+    return s.busy && !ok;
+}
+
+// kLeafUnroll / 2 unchecked updates of one or two orbits.
+template <int NS>
+__device__ __forceinline__ void half_block(float *x, float *y, const float *cr, const float *ci)
+{
+    if (NS == 1) {
+#pragma unroll
+        for (int k = 0; k < kLeafUnroll / 2; ++k)
+            z_update(x[0], y[0], cr[0], ci[0]);
+    } else {
+        f32x2 X = pack2(x[0], x[NS - 1]), Y = pack2(y[0], y[NS - 1]);
+        const f32x2 CR = pack2(cr[0], cr[NS - 1]), CI = pack2(ci[0], ci[NS - 1]);
+#pragma unroll
+        for (int k = 0; k < kLeafUnroll / 2; ++k)
+            z_update2(X, Y, CR, CI);
+        unpack2(X, x[0], x[NS - 1]);
+        unpack2(Y, y[0], y[NS - 1]);
+    }
+}
+
+// One round of the refill loop: an unchecked block of kLeafUnroll updates on
+// the first NS slots (the results of an idle slot are not used), and what
+// follows for each slot (settle_slot).  Once `thr` slots or more are idle or
+// wait, the waiting orbits are parked (the state before the block and the
+// block's midpoint state go to the park buffer), and whenever 32 orbits are
+// parked the warp finishes them together.  Returns whether `thr` was reached.
+template <bool COUNT, bool BATCH, int NS>
+__device__ __forceinline__ bool refill_round(const LeafArgs &a, WarpLeaf<BATCH> &w, WarpFill &f,
+                                             Slot *s, uint32_t thr, uint32_t lane,
+                                             unsigned long long &it, unsigned long long &lpx)
+{
+    float x[NS], y[NS], cr[NS], ci[NS], mx[NS], my[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        x[i] = s[i].x;
+        y[i] = s[i].y;
+        cr[i] = s[i].cr;
+        ci[i] = s[i].ci;
+    }
+    half_block<NS>(x, y, cr, ci);
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        mx[i] = x[i];
+        my[i] = y[i];
+    }
+    half_block<NS>(x, y, cr, ci);
+    bool wait[NS];
+    uint32_t still = 0;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        wait[i] = settle_slot<COUNT, BATCH>(a, s[i], x[i], y[i], it, lpx);
+        still += (uint32_t)__popc(__ballot_sync(kFull, wait[i] || !s[i].busy));
+    }
+    if (still < thr)
+        return false;
+    const unsigned lt = lanes_below();
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        const unsigned p = __ballot_sync(kFull, wait[i]);
+        if (wait[i]) {
+            const uint32_t k = f.parked + (uint32_t)__popc(p & lt);
+            w.park_s[k] = make_float4(s[i].x, s[i].y, mx[i], my[i]);
+            w.park_u[k] = make_uint2(s[i].d, s[i].pix);
+            if (BATCH)
+                w.park_f[k] = s[i].frame;
+            s[i].busy = false;
+        }
+        f.parked += (uint32_t)__popc(p);
+    }
+    __syncwarp();
+    while (f.parked >= 32u) {
+        f.parked -= 32u;
+        const uint32_t k = f.parked + lane;
+        const float4 sv = w.park_s[k];
+        const uint2 uv = w.park_u[k];
+        const uint32_t fr = BATCH ? w.park_f[k] : 0u;
+        __syncwarp();
+        finish_parked<COUNT, BATCH>(a, sv, uv, fr, it);
+        if (COUNT)
+            ++lpx;
+    }
+    return true;
 }
 
 }  // namespace ask

@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 CASES = [
     (1, 50, 1, 2, 1), (2, 50, 1, 2, 4), (7, 63, 1, 2, 8), (33, 64, 1, 2, 64), (97, 65, 3, 2, 32),
     (250, 300, 4, 2, 64), (513, 700, 2, 4, 256), (777, 1, 5, 3, 64), (1000, 40, 16, 2, 32),
+    (256, 2048, 2, 2, 256), (200, 3001, 1, 2, 256),  # orbits that repeat themselves, to odd caps
     (1024, 512, 16, 2, 32), (1025, 129, 1, 2, 2048), (1200, 200, 300, 2, 4),
 ]
 
