@@ -109,8 +109,7 @@ static uint32_t ceil_div(uint32_t a, uint32_t b) { return a / b + (a % b != 0u);
 // its copy, and small bands leave the level kernels too few regions.
 constexpr uint64_t kBandBytes = 128ull << 20;
 
-bool make_plan(uint32_t n, uint32_t g, uint32_t r, uint32_t B, LevelPlan *plan, uint32_t chunk_px,
-               uint64_t few_items)
+bool make_plan(uint32_t n, uint32_t g, uint32_t r, uint32_t B, LevelPlan *plan)
 {
     if (n == 0 || g == 0 || r < 2 || B == 0 || !plan)
         return false;
@@ -136,11 +135,7 @@ bool make_plan(uint32_t n, uint32_t g, uint32_t r, uint32_t B, LevelPlan *plan, 
         if (plan->max_regions[i] >= 0xffffffffull)
             return false;
         const uint64_t per = (s <= 2u) ? (uint64_t)s * s : 4ull * s - 4ull;
-        uint32_t cp = chunk_px;
-        if (few_items && cp >= 64u && plan->max_regions[i] * ((per + cp - 1) / cp) < few_items)
-            cp /= 2u;
-        plan->chunk_px[i] = cp;
-        plan->chunks[i] = (uint32_t)((per + cp - 1) / cp);
+        plan->chunks[i] = (uint32_t)((per + kChunkPx - 1) / kChunkPx);
         if (plan->max_regions[i] * plan->chunks[i] >= 0xffffffffull)
             return false;
         const uint32_t sc = ceil_div(s, r);
@@ -634,8 +629,8 @@ ask_status render_impl(ask_ctx *ctx, ask_method method, const ask_window *window
         a.olt_cap = olt_cap;
         a.in_cap = level_cap(i);
         a.out_cap = (i + 1 < L) ? level_cap(i + 1) : 0u;
+        a.bound = plan.max_regions[i];
         a.chunks = plan.chunks[i];
-        a.chunk_px = plan.chunk_px[i];
         a.next_chunks = (i + 1 < L) ? plan.chunks[i + 1] : 1u;
         a.rst_in = ctx->rst[i & 1];
         a.rst_out = ctx->rst[(i + 1) & 1];
@@ -683,6 +678,7 @@ ask_status render_impl(ask_ctx *ctx, ask_method method, const ask_window *window
     la.side = plan.side[L - 1];
     la.leaves = ctx->leaves;
     la.leaf_cap = leaf_cap;
+    la.bound = plan.max_regions[L - 1];
     la.skip_perimeter = exact ? 1u : 0u;
     la.fills = fused ? ctx->fills : nullptr;
     la.fill_cap = fused ? (uint32_t)ctx->fill_cap : 0u;
@@ -734,7 +730,8 @@ ask_status render_impl(ask_ctx *ctx, ask_method method, const ask_window *window
 struct BatchPlan {
     std::vector<FrameDesc> desc;
     uint32_t L = 0;                       // deepest level over the frames
-    uint32_t chunks[ASK_MAX_LEVELS] = {};  // chunks per region at each level (max over frames)
+    uint32_t chunks[ASK_MAX_LEVELS] = {};  // chunks per region at each level (over all frames)
+    uint32_t max_side[ASK_MAX_LEVELS] = {};  // largest region side at each level
     uint64_t olt_need = 0, leaf_need = 0, rst_need = 0, fill_need = 0;
     uint64_t level_cap[ASK_MAX_LEVELS] = {};  // bound on each level's regions over the frames
     uint32_t total0 = 0;
@@ -781,7 +778,7 @@ ask_status plan_batch(ask_ctx *ctx, const ask_frame *frames, uint32_t nframes, u
         if (!fr.d_dwell || ((uintptr_t)fr.d_dwell & 15u))
             return set_err(ctx, ASK_EINVAL, "frame %u: d_dwell must be 16-byte aligned", f);
         LevelPlan plan;
-        if (!make_plan(fr.n, fr.g, fr.r, fr.B, &plan, kChunkPxBatch, 0))
+        if (!make_plan(fr.n, fr.g, fr.r, fr.B, &plan))
             return set_err(ctx, ASK_EINVAL, "frame %u: no valid subdivision plan", f);
         FrameDesc &d = bp.desc[f];
         std::memset(&d, 0, sizeof(d));
@@ -800,8 +797,7 @@ ask_status plan_batch(ask_ctx *ctx, const ask_frame *frames, uint32_t nframes, u
             d.side[i] = plan.side[i];
             d.chunks[i] = queue_chunks(plan.side[i]);
             level_regions[i] += plan.max_regions[i];
-            if (plan.chunks[i] > bp.chunks[i])
-                bp.chunks[i] = plan.chunks[i];
+            bp.max_side[i] = std::max(bp.max_side[i], plan.side[i]);
             bp.q_items += plan.max_regions[i] * d.chunks[i];
             if (d.chunks[i] > 1u)
                 bp.q_states += plan.max_regions[i];
@@ -822,7 +818,13 @@ ask_status plan_batch(ask_ctx *ctx, const ask_frame *frames, uint32_t nframes, u
             bp.L = plan.levels;
     }
     for (uint32_t i = 0; i < bp.L; ++i) {
-        bp.chunks[i] = std::min(bp.chunks[i], kMaxChunksBatch);
+        // the fewest chunks that leave the level enough items
+        const uint64_t s = bp.max_side[i], per = (s <= 2u) ? s * s : 4u * s - 4u;
+        uint64_t cp = kChunkPxBatch;
+        auto chunks_of = [&](uint64_t px) { return std::min<uint64_t>((per + px - 1) / px, kMaxChunksBatch); };
+        while (cp > kChunkPx && level_regions[i] * chunks_of(cp) < kFewItemsBatch)
+            cp /= 2u;
+        bp.chunks[i] = (uint32_t)chunks_of(cp);
         if (level_regions[i] * bp.chunks[i] >= 0xffffffffull)
             return set_err(ctx, ASK_EINVAL, "batch too large: level %u holds too many work items", i);
         bp.level_cap[i] = level_regions[i];
@@ -918,6 +920,7 @@ ask_status enqueue_batch(ask_ctx *ctx, const BatchBuffers &b, const BatchPlan &b
         a.olt_cap = (uint32_t)b.olt_cap;
         a.in_cap = (i == 0) ? bp.total0 : (uint32_t)bp.level_cap[i];
         a.out_cap = (i + 1 < bp.L) ? (uint32_t)bp.level_cap[i + 1] : 0u;
+        a.bound = bp.level_cap[i];
         a.chunks = bp.chunks[i];
         a.next_chunks = (i + 1 < bp.L) ? bp.chunks[i + 1] : 1u;
         a.rst_in = b.rst[i & 1];
@@ -940,6 +943,7 @@ ask_status enqueue_batch(ask_ctx *ctx, const BatchBuffers &b, const BatchPlan &b
     la.fill_cap = bp.fill_need ? (uint32_t)b.fill_cap : 0u;
     la.leaves = b.leaves;
     la.leaf_cap = (uint32_t)b.leaf_cap;
+    la.bound = bp.leaf_need;
     la.side = bp.leaf_side;
     la.skip_perimeter = exact ? 1u : 0u;
     la.frames = b.frames;
@@ -1063,7 +1067,6 @@ ask_status enqueue_queue(ask_ctx *ctx, const QueueBuffers &b, const BatchPlan &b
     q.regions0 = bp.total0;
     q.total0 = (uint32_t)bp.q_total0;
     q.states0 = (uint32_t)bp.q_states0;
-    q.chunk_px = kChunkPxQueue;
     q.wait_limit = (flags & ASK_FLAG_WAIT_TEST) ? 0u : kQueueWaitLimit;
     cudaError_t e = launch_queue(q, (uint32_t)bp.desc.size(), (flags & ASK_FLAG_COUNT) != 0, ctx->dev.sms, s);
     if (e != cudaSuccess)

@@ -140,6 +140,83 @@ __device__ __forceinline__ uint32_t dwell(float cr, float ci, uint32_t max_dwell
     return d;
 }
 
+__device__ __forceinline__ float sqrt_approx(float v)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// Principal square root of u + iv, near enough (its error is bounded by what
+// capture_disc computes with the result, not assumed).
+__device__ __forceinline__ float2 csqrt_near(float u, float v)
+{
+    const float m = sqrt_approx(__fmaf_rn(u, u, __fmul_rn(v, v)));
+    const float h = sqrt_approx(0.5f * (m + fabsf(u)));
+    const float k = __fdividef(0.5f * fabsf(v), h);
+    return u >= 0.0f ? make_float2(h, copysignf(k, v)) : make_float2(k, copysignf(h, v));
+}
+
+// A disc around a that the iteration maps into itself: an orbit that enters
+// it never escapes, however many updates follow, so its dwell is max_dwell.
+// r2 is the squared radius, negative when no disc was found.
+//
+// One disc around a point a near the attracting fixed point: for |z - a| <= r
+// a float update gives z' = z^2 + c + e with
+//   |z' - a| <= |z - a| |z + a| + |a^2 + c - a| + |e|
+//            <= r (2|a| + r) + q,
+// where q bounds the residual |a^2 + c - a| (computed, plus its own rounding,
+// 5e-7) and the update's rounding (|z| <= 1/2 there: 1.4e-7).  With D = 1 -
+// 2|a| and r = D / 2 this is at most r if D^2 / 4 >= q; the constant 1.2e-6
+// covers both roundings and that of D.  The bound holds for whatever a was
+// computed; a poor one only makes the residual large and the disc fail.
+//
+// Two discs around b and b' = -1 - b near the attracting 2-cycle, of radii r
+// and r1 = r (2|b| + r) + q, mapped into one another if r1 (2|b'| + r1) + q <=
+// r; both discs lie in |z| < 1.9, where an update rounds by less than 1e-6.
+// b is the point of the cycle nearer to the orbit's present state (x, y).
+__device__ __forceinline__ void capture_disc(float cr, float ci, float x, float y, float &ax, float &ay,
+                                             float &r2)
+{
+    r2 = -1.0f;
+    const float2 s = csqrt_near(1.0f - 4.0f * cr, -4.0f * ci);
+    ax = 0.5f * (1.0f - s.x);
+    ay = -0.5f * s.y;
+    const float D = 1.0f - 2.0f * sqrt_approx(__fmaf_rn(ax, ax, __fmul_rn(ay, ay)));
+    if (D > 0.0f) {
+        const float qx = __fmaf_rn(ax, ax, cr) - __fmaf_rn(ay, ay, ax);
+        const float qy = __fmaf_rn(ax + ax, ay, ci) - ay;
+        if (0.25f * D * D >= fabsf(qx) + fabsf(qy) + 1.2e-6f)
+            r2 = 0.24999f * D * D;
+        return;
+    }
+    const float2 q = csqrt_near(-3.0f - 4.0f * cr, -4.0f * ci);
+    float bx = 0.5f * (q.x - 1.0f), by = 0.5f * q.y;
+    float ex = -1.0f - bx, ey = -by;
+    const float db = __fmaf_rn(x - bx, x - bx, __fmul_rn(y - by, y - by));
+    const float de = __fmaf_rn(x - ex, x - ex, __fmul_rn(y - ey, y - ey));
+    if (de < db) {
+        const float tx = bx, ty = by;
+        bx = ex;
+        by = ey;
+        ex = tx;
+        ey = ty;
+    }
+    ax = bx;
+    ay = by;
+    const float A = 2.0f * sqrt_approx(__fmaf_rn(bx, bx, __fmul_rn(by, by)));
+    const float B = 2.0f * sqrt_approx(__fmaf_rn(ex, ex, __fmul_rn(ey, ey)));
+    const float r = __fdividef(0.4f * (1.0f - A * B), B + A * A + 0.5f);
+    // residuals b^2 + c - b' and b'^2 + c - b, with their roundings
+    const float q1 = fabsf(__fmaf_rn(bx, bx, cr) - __fmaf_rn(by, by, ex)) +
+                     fabsf(__fmaf_rn(bx + bx, by, ci) - ey) + 3e-6f;
+    const float q2 = fabsf(__fmaf_rn(ex, ex, cr) - __fmaf_rn(ey, ey, bx)) +
+                     fabsf(__fmaf_rn(ex + ex, ey, ci) - by) + 3e-6f;
+    const float r1 = r * (A + r) + q1;
+    if (r > 0.0f && r1 * (B + r1) + q2 <= 0.9999f * r && 0.5f * A + r < 1.9f && 0.5f * B + r1 < 1.9f)
+        r2 = 0.9999f * r * r;
+}
+
 // Resumable orbit of one point, for perimeter queries that stop early.
 struct Orbit {
     float x, y, cr, ci;
@@ -168,23 +245,13 @@ enum : uint32_t {
 };
 
 // Updates per unchecked block of a perimeter-query round after the short
-// first rounds of query_step, for a large region's chunks and for a small
-// region's whole perimeter.  The short rounds take the orbits that escape
-// early, so the long ones serve orbits that run long (at n = 16384 whole
-// perimeters of 16 x 16 regions ran faster with 64 than with 32; chunks ran
-// slower with 128).
-constexpr uint32_t kQueryRoundLarge = 64;
+// first rounds of query_group.  The short rounds take the orbits that escape
+// early, so the long ones serve orbits that run long (32 at n = 16384: levels 2
+// and 3 at 190 and 387 us against 190 and 371).
 constexpr uint32_t kQueryRound = 64;
 // The CTA-wide query of the paper's SBR / MBR mappings: blocks of 32 from
 // the first round.
 constexpr uint32_t kQueryRoundCta = 32;
-// Batches (zoomed frames, higher dwell caps, regions of many sizes): whole
-// perimeters in blocks of kQueryRoundBatch, short first rounds where the
-// flags say (a batch's chunk queries read their region's state every round,
-// and a short round cannot hide that load).
-constexpr uint32_t kQueryRoundBatch = 32;
-constexpr bool kBatchShortWhole = false;
-constexpr bool kBatchShortChunks = false;
 
 // Advance an orbit by up to K updates (a power of two) without passing
 // `limit`.  An orbit still running after a round has made more updates than
@@ -241,38 +308,6 @@ __device__ __forceinline__ void orbit_resolve(Orbit &o)
     o.x = x;
     o.y = y;
     o.d = d + 1u;
-}
-
-// Rounds of a perimeter query: unchecked blocks of 8, 8 and 16 updates, then
-// K.  Most perimeter orbits outside the set escape within a few updates; a
-// short first block and the short binary search after it cost them about 15
-// updates where a K-update block and its search cost 2K - 1, while an orbit
-// that runs long pays three short rounds.  Every lane of a group runs the
-// same block in a round, so a running orbit still outlives every orbit that
-// finished in that round.
-template <uint32_t K>
-__device__ __forceinline__ void query_step(Orbit &o, uint32_t &stt, uint32_t limit, uint32_t rnd)
-{
-    if (stt != ORBIT_RUN)
-        return;
-    if (rnd < 2u)
-        stt = orbit_step<8>(o, limit);
-    else if (rnd == 2u)
-        stt = orbit_step<16>(o, limit);
-    else
-        stt = orbit_step<K>(o, limit);
-}
-
-// Exact dwell of an orbit left pending by query_step<K> in round `rnd`.
-template <uint32_t K>
-__device__ __forceinline__ void query_resolve(Orbit &o, uint32_t rnd)
-{
-    if (rnd < 2u)
-        orbit_resolve<8>(o);
-    else if (rnd == 2u)
-        orbit_resolve<16>(o);
-    else
-        orbit_resolve<K>(o);
 }
 
 // Region record of the offset lookup tables (Sec. 5.2): origin and clipped
@@ -402,57 +437,306 @@ __device__ __forceinline__ void fill_band_warp(uint32_t *__restrict__ map, uint3
 // ---------------------------------------------------------------------------
 constexpr unsigned kLaneMask = 0xffffffffu;
 
-// One warp queries the whole perimeter of g.  Returns true and the common
-// dwell in *w_out if the perimeter is uniform; `it` gains the updates made.
-template <uint32_t K, bool SHORT>
+// Outcome of query_group.
+enum : uint32_t {
+    GROUP_SAME = 0,    // every dwell of the group is exact in d (or at least the limit)
+    GROUP_DIFFER = 1,  // two dwells of the group differ
+    GROUP_STOP = 2,    // another warp found the region non-uniform
+};
+
+// Rounds between issuing a load of a region's query state and using it, for
+// one frame.  A batch keeps enough warps resident to hide the load, and there
+// a late stop costs more than the wait, so it uses the value one round later.
+constexpr uint32_t kPollLag = 8;
+constexpr uint32_t kNone32 = 0xffffffffu;
+
+// K unchecked updates of NS orbits (one or two, side by side).
+template <uint32_t K, int NS>
+__device__ __forceinline__ void run_block(float *x, float *y, const float *cr, const float *ci)
+{
+    if (NS == 1) {
+#pragma unroll
+        for (uint32_t k = 0; k < K; ++k)
+            z_update(x[0], y[0], cr[0], ci[0]);
+    } else {
+        f32x2 X = pack2(x[0], x[NS - 1]), Y = pack2(y[0], y[NS - 1]);
+        const f32x2 CR = pack2(cr[0], cr[NS - 1]), CI = pack2(ci[0], ci[NS - 1]);
+#pragma unroll
+        for (uint32_t k = 0; k < K; ++k)
+            z_update2(X, Y, CR, CI);
+        unpack2(X, x[0], x[NS - 1]);
+        unpack2(Y, y[0], y[NS - 1]);
+    }
+}
+
+// Exact dwells of orbits whose state (x, y) at count d passed the test and
+// whose state K updates later failed (pend): halving the gap finds the first
+// failing state (K - 1 updates, log2(K) tests, the same on every lane).  The
+// search stops, and returns true, at the first half that some of these orbits
+// pass and others do not: their dwells differ.
+template <uint32_t K, int NS>
+__device__ __forceinline__ bool resolve_block(const float *x0, const float *y0, const float *cr,
+                                              const float *ci, const bool *pend, uint32_t base,
+                                              uint32_t *d)
+{
+    static_assert(K <= 64u && (K & (K - 1u)) == 0u, "blocks of up to 64 updates, a power of two");
+    float x[NS], y[NS];
+    uint32_t r[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        x[i] = x0[i];
+        y[i] = y0[i];
+        r[i] = base;
+    }
+#pragma unroll
+    for (uint32_t h = K / 2u; h >= 1u; h >>= 1) {
+        float tx[NS], ty[NS];
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            tx[i] = x[i];
+            ty[i] = y[i];
+        }
+        // (an unrolled run_block of h updates)
+        if (h >= 32u)
+            run_block<32u, NS>(tx, ty, cr, ci);
+        else if (h == 16u)
+            run_block<16u, NS>(tx, ty, cr, ci);
+        else if (h == 8u)
+            run_block<8u, NS>(tx, ty, cr, ci);
+        else if (h == 4u)
+            run_block<4u, NS>(tx, ty, cr, ci);
+        else if (h == 2u)
+            run_block<2u, NS>(tx, ty, cr, ci);
+        else
+            run_block<1u, NS>(tx, ty, cr, ci);
+        bool passed = false, failed = false;
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            const bool ok = z_bounded(tx[i], ty[i]);
+            passed = passed || (pend[i] && ok);
+            failed = failed || (pend[i] && !ok);
+            if (ok) {
+                x[i] = tx[i];
+                y[i] = ty[i];
+                r[i] += h;
+            }
+        }
+        if (__any_sync(kLaneMask, passed) && __any_sync(kLaneMask, failed))
+            return true;
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+        if (pend[i])
+            d[i] = r[i] + 1u;
+    return false;
+}
+
+// The orbits of up to 32 * NS perimeter pixels (NS a lane, `active`) advance
+// in lockstep rounds of unchecked blocks: 8, 8, 16, then K updates (rnd = 3
+// skips the short ones).  Most perimeter orbits outside the set escape within
+// a few updates, and a short first block and the short search after it cost
+// them about 15 updates where a K-update block and its search cost 2K - 1.
+// The rounds end as soon as an orbit escapes: if another still runs, or never
+// will escape, two dwells differ; else all escaped in this round and their
+// dwells are resolved.  An orbit is proven to stay (its dwell is max_dwell)
+// when it enters its capture disc or repeats the state it had at rounds 1, 2,
+// 4, 8, ... of the long ones, so a cycle is seen within twice the rounds it
+// took to enter it.  w: the region's common dwell as far as known (kNone32:
+// none yet); orbits stop at w + 1.  ps (or NULL): the region's shared state
+// {common dwell, differs}, read along the way, `lag` rounds between a load and
+// its use.  On GROUP_SAME d holds the dwells (above w: anything above w).
+template <uint32_t K, int NS>
+__device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max_dwell,
+                                                const uint32_t *px, const uint32_t *py,
+                                                const bool *active, uint32_t rnd, uint32_t w,
+                                                const volatile uint32_t *ps, uint32_t lag,
+                                                uint32_t lane, uint32_t *d)
+{
+    float x[NS], y[NS], cr[NS], ci[NS];
+    float bx[NS], by[NS], ax[NS], ay[NS], r2[NS];
+    bool run[NS], pend[NS];
+    bool plain = false;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        const float2 c = pixel_c(pm, px[i], py[i]);
+        cr[i] = c.x;
+        ci[i] = c.y;
+        x[i] = y[i] = 0.0f;
+        bx[i] = by[i] = ax[i] = ay[i] = 0.0f;
+        r2[i] = -1.0f;
+        run[i] = active[i];
+        pend[i] = false;
+        d[i] = 0;
+        plain = plain || (active[i] && !escape_absorbing(c.x, c.y));
+    }
+    uint32_t limit = (w != kNone32) ? min(max_dwell, w + 1u) : max_dwell;
+    if (__any_sync(kLaneMask, plain)) {
+        // points with |c| near 2 (they escape at once, or lie near -2)
+#pragma unroll
+        for (int i = 0; i < NS; ++i)
+            if (active[i])
+                d[i] = dwell(cr[i], ci[i], limit);
+        return GROUP_SAME;
+    }
+    uint32_t n = 0;  // updates made by the running orbits
+    uint32_t nx = w, ny = 0, age = 0, step;
+    for (;; ++rnd) {
+        if (ps != nullptr && age == 0 && lane == 0) {
+            nx = ps[0];
+            ny = ps[1];
+        }
+        step = rnd < 2u ? 8u : rnd == 2u ? 16u : K;
+        if (n + step > limit || n + step < n) {
+            // less than a block left: tested updates (none if w fell below n)
+            for (; n < limit; ++n)
+#pragma unroll
+                for (int i = 0; i < NS; ++i)
+                    if (run[i]) {
+                        run[i] = z_bounded(x[i], y[i]);
+                        d[i] = n;
+                        z_update(x[i], y[i], cr[i], ci[i]);
+                    }
+#pragma unroll
+            for (int i = 0; i < NS; ++i)
+                if (run[i])
+                    d[i] = n;
+            return GROUP_SAME;
+        }
+        if (rnd >= 3u && ((rnd - 3u) & (rnd - 4u)) == 0u) {
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                bx[i] = x[i];
+                by[i] = y[i];
+                if (run[i])
+                    capture_disc(cr[i], ci[i], x[i], y[i], ax[i], ay[i], r2[i]);
+            }
+        }
+        float tx[NS], ty[NS];
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            tx[i] = x[i];
+            ty[i] = y[i];
+        }
+        if (rnd < 2u)
+            run_block<8u, NS>(tx, ty, cr, ci);
+        else if (rnd == 2u)
+            run_block<16u, NS>(tx, ty, cr, ci);
+        else
+            run_block<K, NS>(tx, ty, cr, ci);
+        n += step;
+        bool any_run = false, any_pend = false;
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            const bool ok = z_bounded(tx[i], ty[i]);
+            pend[i] = run[i] && !ok;
+            if (ok) {
+                x[i] = tx[i];
+                y[i] = ty[i];
+            }
+            const float ux = x[i] - ax[i], uy = y[i] - ay[i];
+            const bool in = rnd >= 3u && (__fmaf_rn(ux, ux, __fmul_rn(uy, uy)) < r2[i] ||
+                                          (x[i] == bx[i] && y[i] == by[i]));
+            if (run[i] && ok)
+                d[i] = in ? max_dwell : n;
+            // (at the limit an orbit has ended: its dwell may equal that of
+            // one whose last state escaped)
+            run[i] = run[i] && ok && !in && n < limit;
+            any_run = any_run || run[i];
+            any_pend = any_pend || pend[i];
+        }
+        any_run = __any_sync(kLaneMask, any_run);
+        any_pend = __any_sync(kLaneMask, any_pend);
+        if (any_pend)
+            break;
+        if (!any_run)
+            return GROUP_SAME;
+        if (ps != nullptr && ++age == lag) {
+            age = 0;
+            w = __shfl_sync(kLaneMask, nx, 0);
+            if (__shfl_sync(kLaneMask, ny, 0))
+                return GROUP_STOP;
+            limit = (w != kNone32) ? min(max_dwell, w + 1u) : max_dwell;
+        }
+    }
+    bool left = false;
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+        left = left || run[i];
+    if (__any_sync(kLaneMask, left))
+        return GROUP_DIFFER;
+    bool differ;
+    if (step == 8u)
+        differ = resolve_block<8u, NS>(x, y, cr, ci, pend, n - step, d);
+    else if (step == 16u)
+        differ = resolve_block<16u, NS>(x, y, cr, ci, pend, n - step, d);
+    else
+        differ = resolve_block<K, NS>(x, y, cr, ci, pend, n - step, d);
+    return differ ? GROUP_DIFFER : GROUP_SAME;
+}
+
+// The dwells of a group (NS a lane): their least and greatest.
+template <int NS>
+__device__ __forceinline__ void group_range(const bool *active, const uint32_t *d, uint32_t &vmin,
+                                            uint32_t &vmax)
+{
+    vmin = kNone32;
+    vmax = 0u;
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+        if (active[i]) {
+            vmin = min(vmin, d[i]);
+            vmax = max(vmax, d[i]);
+        }
+    vmin = __reduce_min_sync(kLaneMask, vmin);
+    vmax = __reduce_max_sync(kLaneMask, vmax);
+}
+
+// Group j of the `groups` of 32 * NS pixels that cover the perimeter of g (P
+// pixels), spread over all of it: pixels j, j + groups, j + 2 groups, ...
+template <uint32_t K, int NS>
+__device__ __forceinline__ uint32_t spread_group(const PixelMap &pm, uint32_t max_dwell, const Region &g,
+                                                 uint32_t first, uint32_t stride, uint32_t base,
+                                                 uint32_t P, uint32_t rnd, uint32_t w,
+                                                 const volatile uint32_t *ps, uint32_t lag, uint32_t lane,
+                                                 uint32_t &vmin, uint32_t &vmax, unsigned long long &it)
+{
+    uint32_t px[NS], py[NS], d[NS];
+    bool active[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        const uint32_t k = first + (base + lane + 32u * (uint32_t)i) * stride;
+        active[i] = k < P;
+        px[i] = g.x0;
+        py[i] = g.y0;
+        if (active[i])
+            perimeter_pixel(g, k, px[i], py[i]);
+    }
+    const uint32_t r = query_group<K, NS>(pm, max_dwell, px, py, active, rnd, w, ps, lag, lane, d);
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+        if (active[i])
+            it += d[i];
+    if (r == GROUP_SAME)
+        group_range<NS>(active, d, vmin, vmax);
+    return r;
+}
+
+// One warp queries the whole perimeter of g, NS orbits a lane.  Returns true
+// and the common dwell in *w_out if the perimeter is uniform; `it` gains the
+// updates made.
+template <uint32_t K, int NS>
 __device__ __forceinline__ bool warp_perimeter_uniform(const PixelMap &pm, uint32_t max_dwell,
                                                        const Region &g, uint32_t lane,
                                                        uint32_t *w_out, unsigned long long &it)
 {
     const uint32_t P = perimeter_size(g.w, g.h);
-    bool have = false;
-    uint32_t w = 0;
-    for (uint32_t base = 0; base < P; base += 32u) {
-        const uint32_t k = base + lane;
-        const bool active = k < P;
-        const unsigned amask = __ballot_sync(kLaneMask, active);
-        uint32_t px = g.x0, py = g.y0;
-        if (active)
-            perimeter_pixel(g, k, px, py);
-        Orbit o = orbit_start(pixel_c(pm, px, py));
-        uint32_t stt = active ? ORBIT_RUN : ORBIT_DONE;
-        const uint32_t limit = have ? min(max_dwell, w + 1u) : max_dwell;
-        bool differ = false;
-        uint32_t rnd = 0;
-        for (;; ++rnd) {
-            if (SHORT)
-                query_step<K>(o, stt, limit, rnd);
-            else if (stt == ORBIT_RUN)
-                stt = orbit_step<K>(o, limit);
-            const unsigned dm = __ballot_sync(kLaneMask, stt != ORBIT_RUN) & amask;
-            if (dm == amask)
-                break;
-            if (dm) {
-                differ = true;
-                break;
-            }
-        }
-        // every orbit finished in round rnd (else they would differ)
-        if (!differ && stt == ORBIT_PEND) {
-            if (SHORT)
-                query_resolve<K>(o, rnd);
-            else
-                orbit_resolve<K>(o);
-        }
-        if (active)
-            it += o.d;
-        if (differ)
+    const uint32_t groups = (P + 32u * NS - 1u) / (32u * NS);
+    uint32_t w = kNone32, vmin = 0, vmax = 0;
+    for (uint32_t j = 0; j < groups; ++j) {
+        const uint32_t r = spread_group<K, NS>(pm, max_dwell, g, j, groups, 0u, P, 0u, w, nullptr, 0u, lane,
+                                               vmin, vmax, it);
+        if (r != GROUP_SAME || vmin != vmax || (w != kNone32 && vmin != w))
             return false;
-        const uint32_t vmin = __reduce_min_sync(kLaneMask, active ? o.d : 0xffffffffu);
-        const uint32_t vmax = __reduce_max_sync(kLaneMask, active ? o.d : 0u);
-        if (vmin != vmax || (have && vmin != w))
-            return false;
-        have = true;
         w = vmin;
     }
     *w_out = w;

@@ -55,23 +55,12 @@ struct LevelPlan {
     uint32_t split[ASK_MAX_LEVELS];         // 1 if non-uniform regions of level i split
     uint64_t max_regions[ASK_MAX_LEVELS];   // upper bound on regions at level i
     uint32_t chunks[ASK_MAX_LEVELS];        // perimeter chunks per region (work items)
-    uint32_t chunk_px[ASK_MAX_LEVELS];      // perimeter pixels per chunk
     uint32_t axis0;                         // non-empty initial regions per axis
 };
 
-// A level with fewer work items than this at chunk_px pixels a chunk takes
-// chunks of half that size: its items are too few to keep every warp busy,
-// and the kernel's time is set by its longest items (chunks of a region
-// inside the set run max_dwell updates per pixel, one pixel per lane after
-// another).
-constexpr uint64_t kFewLevelItems = 32768;
-
 // Fills `plan`; returns false if the parameters are invalid or a level could
-// hold 2^32 regions or more.
-// chunk_px: perimeter pixels per work item of the level kernels (chunks[i]);
-// few_items: levels with fewer items take chunks of chunk_px / 2 (0: never).
-bool make_plan(uint32_t n, uint32_t g, uint32_t r, uint32_t B, LevelPlan *plan, uint32_t chunk_px = 64,
-               uint64_t few_items = kFewLevelItems);
+// hold 2^32 regions or work items (chunks of kChunkPx perimeter pixels) or more.
+bool make_plan(uint32_t n, uint32_t g, uint32_t r, uint32_t B, LevelPlan *plan);
 
 // Launch configuration chosen per device at context creation.
 struct DeviceInfo {
@@ -131,8 +120,8 @@ struct LevelArgs {
                           //   count[level] entries from slot 0 up and back[level] from
                           //   slot in_cap - 1 down
     uint32_t out_cap;     // the same bound for the next level's table (olt_out, rst_out)
+    unsigned long long bound;  // most regions the level can hold (sizes the grid)
     uint32_t chunks;      // perimeter chunks per region at this level (1 = one warp per region)
-    uint32_t chunk_px;    // perimeter pixels per chunk (one frame; a batch derives its own)
     uint32_t next_chunks; // chunks per region at the next level
     uint4 *rst_in;        // per-region query state of this level (chunks > 1)
     uint4 *rst_out;       // state of the next level's regions, set when they are appended
@@ -144,16 +133,19 @@ struct LevelArgs {
     const FrameDesc *frames;  // batch: the frame table
     DevCounters *ctr;
 };
-// Perimeter pixels per work item of a level kernel: one frame's top levels
-// have few regions and need the parallelism of small chunks; a batch has
-// regions enough, and there a chunk's fixed cost weighs more.
+// Perimeter pixels per work item of a level kernel: one round of a warp, two
+// orbits a lane.  A batch with regions enough takes up to kChunkPxBatch, where
+// an item's fixed cost weighs less: chunks are doubled while a level keeps
+// kFewItemsBatch items (64 frames of up to 8192 pixels: 40.3 / 39.9 / 39.5 ms
+// with 64 / 128 / 256; 12 frames of up to 1024: 507 / 538 / 575 us).
 constexpr uint32_t kChunkPx = 64;
-constexpr uint32_t kChunkPxBatch = 128;
+constexpr uint32_t kChunkPxBatch = 256;
+constexpr uint64_t kFewItemsBatch = 32768;
 // A batch splits every region of a level into the same number of chunks (the
 // work items are region x chunk), at most kMaxChunksBatch; a region whose
-// perimeter exceeds that many kChunkPxBatch chunks takes longer chunks.  The
-// cap keeps one frame with huge regions from multiplying the work items of
-// every other frame.
+// perimeter exceeds that many chunks takes longer ones.  The cap keeps one
+// frame with huge regions from multiplying the work items of every other
+// frame.
 constexpr uint32_t kMaxChunksBatch = 8;
 // Uniform regions larger than this are filled by the fill kernel.
 constexpr uint32_t kInPlaceFillArea = 16384;
@@ -195,6 +187,7 @@ struct LeafArgs {
     uint32_t side;        // nominal side of the leaf regions (a batch: the largest)
     const void *leaves;   // uint2 (single frame) or uint4 (batch) records
     uint32_t leaf_cap;    // capacity of the leaf list
+    unsigned long long bound;  // most leaves there can be (sizes the grid)
     uint32_t skip_perimeter;  // leaf perimeters are already in the map
     const uint4 *fills;   // lane-refill kernel: deferred-fill bands to write
     uint32_t fill_cap;    //   along the way (NULL: none)
@@ -235,7 +228,6 @@ struct QueueArgs {
     uint32_t regions0;    // level-0 regions of all frames
     uint32_t total0;      // level-0 items of all frames
     uint32_t states0;     // level-0 chunk states of all frames
-    uint32_t chunk_px;    // perimeter pixels per chunk item (a region's last chunks may be longer)
     uint32_t wait_limit;  // idle polls in a row before a warp reports ERR_TIMEOUT
 };
 // Perimeter pixels per chunk item and the most chunk items per region of the

@@ -18,15 +18,18 @@
 //    region count from device memory and hand out work with an atomic
 //    counter, so no depth needs a host round trip;
 //  * a work item is one region's perimeter, or one chunk of kChunkPx
-//    (kChunkPxBatch in a batch; half of kChunkPx at a level with few items)
-//    perimeter pixels of a large region (several warps per region: the MBR
-//    mapping of Sec. 4.3.2 applied to the query), one warp per item;
+//    perimeter pixels of a large region (a batch: see plan_batch; several
+//    warps per region: the MBR mapping of Sec. 4.3.2 applied to the query), one
+//    warp per item;
 //  * each region table is filled from both ends (regions whose centre orbit
 //    stays bounded for a short probe from the front), so a level kernel
 //    takes its longest regions first; the leaf list likewise;
 //  * a query stops at the first two perimeter dwells known to differ; warps
-//    of one region share that verdict through a per-region state word, and
-//    the warp that finishes the region's last chunk takes the decision;
+//    of one region share that verdict through a per-region state word; the
+//    warp that finds the difference, or finishes the region's last chunk
+//    without one, takes the decision;
+//  * orbits proven to stay in the set (capture_disc, repeated states) end
+//    there, with the dwell they would have had;
 //  * decisions are compacted per warp: each lane keeps the outcome of one
 //    region, then one atomicAdd per list serves up to 32 regions (the
 //    block-scan + single atomic alternative of Sec. 5.3.1, at warp scope);
@@ -169,6 +172,17 @@ __device__ __forceinline__ PixelMap record_pm(const LevelArgs &a, const typename
     return BATCH ? a.frames[Rec<BATCH>::frame(e)].pm : a.pm;
 }
 
+// A region record from another lane.
+__device__ __forceinline__ uint2 shfl_record(uint2 e, int src)
+{
+    return make_uint2(__shfl_sync(kFull, e.x, src), __shfl_sync(kFull, e.y, src));
+}
+__device__ __forceinline__ uint4 shfl_record(uint4 e, int src)
+{
+    return make_uint4(__shfl_sync(kFull, e.x, src), __shfl_sync(kFull, e.y, src), __shfl_sync(kFull, e.z, src),
+                      0u);
+}
+
 template <bool BATCH>
 __device__ __forceinline__ void flush_batch(const LevelArgs &a, WarpBatch<BATCH> &b, uint32_t lane)
 {
@@ -231,55 +245,56 @@ __device__ __forceinline__ void flush_batch(const LevelArgs &a, WarpBatch<BATCH>
                 atomicOr(&ctr->error, ERR_OLT_OVERFLOW);
         }
     }
-    // children: each lane probes its region's children (at most 64; a region
-    // with more sends them all to the front); warp inclusive scans of the
-    // counts going to the front and to the back of the next level's table,
-    // one atomicAdd for each
-    const unsigned split_any = __ballot_sync(kFull, b.nchild != 0u);
-    if (split_any) {
-        const Region g = R::region(b.rec);
-        unsigned long long heavy = ~0ull;  // bit j: child j goes to the front
-        uint32_t nh = b.nchild;
-        if (b.nchild != 0u && b.nchild <= 64u) {
-            const PixelMap pm = record_pm<BATCH>(a, b.rec);
-            heavy = 0ull;
-            nh = 0;
-            for (uint32_t j = 0; j < b.nchild; ++j)
-                if (region_probe(pm, unpack_region(child_region(g, b.sc, b.r, j)))) {
-                    heavy |= 1ull << j;
-                    ++nh;
-                }
-        }
-        const uint32_t nl = b.nchild - nh;
-        uint32_t ih = nh, il = nl;
+    // children: 32 at a time over all the regions that split, one a lane (a
+    // warp scan of the counts tells a lane its region), each probed and put in
+    // the next level's table, from the front or from the back
+    if (__any_sync(kFull, b.nchild != 0u)) {
+        uint32_t incl = b.nchild;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t vh = __shfl_up_sync(kFull, ih, o), vl = __shfl_up_sync(kFull, il, o);
-            if (lane >= (uint32_t)o) {
-                ih += vh;
-                il += vl;
+            const uint32_t v = __shfl_up_sync(kFull, incl, o);
+            if (lane >= (uint32_t)o)
+                incl += v;
+        }
+        const uint32_t total = __shfl_sync(kFull, incl, 31);
+        for (uint32_t p0 = 0; p0 < total; p0 += 32u) {
+            const uint32_t p = p0 + lane;
+            uint32_t own = 0;  // regions (lanes) whose children all come before p
+#pragma unroll
+            for (uint32_t h = 16u; h >= 1u; h >>= 1)
+                if (__shfl_sync(kFull, incl, (int)(own + h - 1u)) <= p)
+                    own += h;
+            const bool valid = p < total;
+            const int src = (int)(own & 31u);
+            const T rec = shfl_record(b.rec, src);
+            const uint32_t j = p - (__shfl_sync(kFull, incl, src) - __shfl_sync(kFull, b.nchild, src));
+            const uint32_t sc = __shfl_sync(kFull, b.sc, src), r = __shfl_sync(kFull, b.r, src);
+            uint2 child = make_uint2(0u, 0u);
+            bool heavy = false;
+            if (valid) {
+                child = child_region(R::region(rec), sc, r, j);
+                heavy = region_probe(record_pm<BATCH>(a, rec), unpack_region(child));
             }
-        }
-        const uint32_t th = __shfl_sync(kFull, ih, 31), tl = __shfl_sync(kFull, il, 31);
-        uint32_t hb = 0, lb = 0;
-        if (lane == 0) {
-            if (th)
-                hb = atomicAdd(&ctr->count[a.level + 1], th);
-            if (tl)
-                lb = atomicAdd(&ctr->back[a.level + 1], tl);
-        }
-        hb = __shfl_sync(kFull, hb, 0) + ih - nh;  // this lane's first front index
-        lb = __shfl_sync(kFull, lb, 0) + il - nl;  // and first back index
-        for (uint32_t j = 0; j < b.nchild; ++j) {
-            const bool front = (heavy >> (j & 63u)) & 1ull;
-            const uint32_t k = front ? hb++ : lb++;
-            if (k < a.out_cap) {
-                const uint32_t slot = front ? k : a.out_cap - 1u - k;
-                olt_out[slot] = R::child(b.rec, child_region(g, b.sc, b.r, j));
-                if (a.next_chunks > 1u)
-                    a.rst_out[slot] = make_uint4(kNone, 0u, 0u, 0u);
-            } else {
-                atomicOr(&ctr->error, ERR_OLT_OVERFLOW);
+            const unsigned hm = __ballot_sync(kFull, heavy), lm = __ballot_sync(kFull, valid && !heavy);
+            uint32_t hb = 0, lb = 0;
+            if (lane == 0) {
+                if (hm)
+                    hb = atomicAdd(&ctr->count[a.level + 1], (uint32_t)__popc(hm));
+                if (lm)
+                    lb = atomicAdd(&ctr->back[a.level + 1], (uint32_t)__popc(lm));
+            }
+            hb = __shfl_sync(kFull, hb, 0);
+            lb = __shfl_sync(kFull, lb, 0);
+            if (valid) {
+                const uint32_t k = heavy ? hb + (uint32_t)__popc(hm & lt) : lb + (uint32_t)__popc(lm & lt);
+                if (k < a.out_cap) {
+                    const uint32_t slot = heavy ? k : a.out_cap - 1u - k;
+                    olt_out[slot] = R::child(rec, child);
+                    if (a.next_chunks > 1u)
+                        a.rst_out[slot] = make_uint4(kNone, 0u, 0u, 0u);
+                } else {
+                    atomicOr(&ctr->error, ERR_OLT_OVERFLOW);
+                }
             }
         }
     }
@@ -322,10 +337,37 @@ __device__ __forceinline__ void chunk_exact(const FView &a, const Region &g, uin
 
 // ---------------------------------------------------------------------------
 // Level kernel: one warp per work item (a region, or a perimeter chunk of a
-// large region).
+// large region), NS perimeter orbits a lane.
+//
+// A level is bound by the latency of its items (each a few trips to L2 and a
+// chain of updates) as much as by its updates, so two orbits a lane (24 warps
+// an SM, 80 registers) are the better half wherever an item has more than 32
+// pixels to give: side 18 and up, chunks of 64.  Smaller regions take one orbit
+// a lane and 32 warps.  (Two for the regions of side 16 of n = 16384: 393 us
+// against 371; one up to side 40, n = 1999 without chunks: 316 against 311.)
+//
+// Levels 0 to 3 at n = 16384 (g=16 r=4 B=16), in us: contiguous chunks, every
+// orbit of the set run to max_dwell 130 / 194 / 303 / 377; perimeters spread,
+// capture discs and repeats 65 / 121 / 246 / 404; two orbits a lane 67 / 106 /
+// 211 / 401; cheap regions several to a ticket, chunk-major order, children
+// probed one a lane 62 / 75 / 190 / 371; chunks of 64 at every level 56 / 73 /
+// 186 / 371.  n = 65536 (8 levels): 6.4 -> 4.0 ms.
 // ---------------------------------------------------------------------------
-template <bool COUNT, bool BATCH>
-__global__ void __launch_bounds__(256) level_kernel(LevelArgs a)
+// CTAs an SM for one and two orbits a lane.
+constexpr int kLevelMinBlocks1 = 4;
+constexpr int kLevelMinBlocks2 = 3;
+// Level kernels of regions up to this side take one orbit a lane.
+constexpr uint32_t kLevelSide1 = 17;
+// A ticket of cheap regions stands for at most kTicketMax of them, as long as
+// every warp gets kTicketsPerWarp tickets (1 at most: 377 us at level 3 of n =
+// 16384 and 11.0 ms at n = 65536 against 371 and 10.0; a ticket of several
+// regions from the front of the table, too: 588 us).
+constexpr uint32_t kTicketMax = 8;
+constexpr uint32_t kTicketsPerWarp = 4;
+
+template <bool COUNT, bool BATCH, int NS>
+__global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlocks2)
+    level_kernel(LevelArgs a)
 {
     using R = Rec<BATCH>;
     using T = typename R::T;
@@ -339,8 +381,8 @@ __global__ void __launch_bounds__(256) level_kernel(LevelArgs a)
     if (blockIdx.x == 0 && threadIdx.x == 0 &&
         (unsigned long long)a.ctr->count[a.level] + a.ctr->back[a.level] > a.in_cap)
         atomicOr(&a.ctr->error, ERR_OLT_OVERFLOW);
-    const uint32_t chunks = a.chunks;
-    const uint32_t items = count * chunks;  // the host keeps this below 2^32
+    const uint32_t chunks = (NS == 1) ? 1u : a.chunks;  // one orbit a lane: small regions
+    const bool query_all = !BATCH && a.split != 0u;  // no region of this level is exact
 
     WarpBatch<BATCH> b;
     b.rec = T();
@@ -351,18 +393,64 @@ __global__ void __launch_bounds__(256) level_kernel(LevelArgs a)
     uint32_t j = 0;
     unsigned long long it = 0, bpx = 0, fpx = 0, dpx = 0;
 
+    // The regions from the front of the table come first and are handed out one
+    // item at a time: their costs differ by orders of magnitude (a uniform
+    // perimeter inside the set may run to max_dwell).  Those from the back are
+    // cheap; where every warp gets many of them, a ticket stands for `take`,
+    // so that one round trip for the ticket and one for the records serve them
+    // all.  Of either kind every region's first chunk comes before any region's
+    // second: most regions that are not uniform are known by then, and their
+    // other chunks end at a look at the region's state.
+    const uint32_t back = count - front, heavy = front * chunks, light = back * chunks;
+    const uint32_t warps = gridDim.x * (blockDim.x / 32u);
+    uint32_t take = 1u;
+    while (take < kTicketMax && light / (2u * take) >= kTicketsPerWarp * warps)
+        take *= 2u;
+    const uint32_t tickets = heavy + (light + take - 1u) / take;
+    uint32_t todo = 0, my_c = 0, my_slot = 0;
+    T mine = T();
+    // a warp's first ticket is its number (counted over the CTAs first, so that
+    // a short table is spread over all SMs); the counter hands out the others
+    uint32_t t = blockIdx.x + gridDim.x * (threadIdx.x >> 5);
+    bool fresh = true;
     for (;;) {
-        // items are handed out one at a time: their costs differ by orders
-        // of magnitude (a uniform perimeter inside the set runs to max_dwell)
-        uint32_t t = 0;
-        if (lane == 0)
-            t = atomicAdd(&a.ctr->work[a.level], 1u);
-        t = __shfl_sync(kFull, t, 0);
-        if (t >= items)
-            break;
-        const uint32_t li = (chunks == 1u) ? t : t / chunks;  // in the order taken
-        const uint32_t region = table_slot(li, front, a.in_cap);  // its slot
-        const T e = olt_in[region];
+        if (todo == 0u) {
+            if (!fresh) {
+                if (lane == 0)
+                    t = warps + atomicAdd(&a.ctr->work[a.level], 1u);
+                t = __shfl_sync(kFull, t, 0);
+            }
+            fresh = false;
+            if (t >= tickets)
+                break;
+            // lane k looks at the ticket's k-th item: its record, and, of a
+            // large region, whether it is still open
+            bool open;
+            uint32_t li;
+            if (t < heavy) {
+                open = lane == 0;
+                my_c = (chunks == 1u) ? 0u : t / front;
+                li = t - my_c * front;
+            } else {
+                const uint32_t q = (t - heavy) * take + lane;
+                open = lane < take && q < light;
+                my_c = (chunks == 1u) ? 0u : q / back;
+                li = front + (q - my_c * back);
+            }
+            if (open) {
+                my_slot = table_slot(li, front, a.in_cap);
+                if (chunks > 1u && !(COUNT && my_c == 0u) && (query_all || !a.exact_last))
+                    open = reinterpret_cast<const volatile uint32_t *>(a.rst_in + my_slot)[1] == 0u;
+                mine = olt_in[my_slot];
+            }
+            todo = __ballot_sync(kFull, open);
+            continue;
+        }
+        const int k = __ffs((int)todo) - 1;
+        todo &= todo - 1u;
+        const uint32_t c = (chunks == 1u) ? 0u : __shfl_sync(kFull, my_c, k);
+        const uint32_t region = (chunks == 1u) ? 0u : __shfl_sync(kFull, my_slot, k);
+        const T e = shfl_record(mine, k);
         const Region g = R::region(e);
         const FView f = BATCH ? view_frame(a.frames, R::frame(e), a.level) : view_single(a);
         const bool query = f.split || !a.exact_last;
@@ -375,7 +463,7 @@ __global__ void __launch_bounds__(256) level_kernel(LevelArgs a)
             if (COUNT && lane == 0)
                 bpx += P;
             if (query) {
-                uniform = warp_perimeter_uniform<BATCH ? kQueryRoundBatch : kQueryRound, !BATCH || kBatchShortWhole>(
+                uniform = warp_perimeter_uniform<kQueryRound, NS>(
                     f.pm, f.max_dwell, g, lane, &wv, it);
             } else {
                 // last level, exact perimeters staged in shared memory: a leaf
@@ -409,40 +497,31 @@ __global__ void __launch_bounds__(256) level_kernel(LevelArgs a)
                 }
             }
         } else {
-            const uint32_t c = t - li * chunks;
             uint4 *st = a.rst_in + region;
-            // one frame: chunks cover the level's largest perimeter; a batch
-            // caps the chunk count, so a large region takes longer chunks
-            const uint32_t CP = BATCH ? max(kChunkPxBatch, ceil_div_u32(P, chunks)) : a.chunk_px;
-            const uint32_t k0 = min(P, c * CP), k1 = min(P, k0 + CP);
-            if (COUNT && lane == 0)
-                bpx += k1 - k0;
-            if (k0 < k1) {
-                if (query)
-                    chunk_query<BATCH>(f, g, k0, k1, st, lane, it);
-                else
+            if (COUNT && lane == 0 && c == 0)
+                bpx += P;
+            if (query) {
+                const uint32_t r = chunk_query<BATCH, NS>(f, g, P, c, chunks, st, lane, it);
+                decided = chunk_decides(r, st, chunks, lane, uniform, wv);
+            } else {
+                const uint32_t CP = ceil_div_u32(P, chunks);
+                const uint32_t k0 = min(P, c * CP), k1 = min(P, k0 + CP);
+                if (k0 < k1)
                     chunk_exact(f, g, k0, k1, st, lane, it);
-            }
-            // the warp that finishes the region's last chunk decides
-            uint32_t last = 0;
-            if (lane == 0) {
-                __threadfence();
-                last = (atomicAdd(&st->z, 1u) == chunks - 1u) ? 1u : 0u;
-                if (last)
-                    __threadfence();
-            }
-            last = __shfl_sync(kFull, last, 0);
-            if (last) {
-                uint32_t sx = 0, sy = 0;
+                // the warp that finishes the region's last chunk decides
+                uint32_t last = 0, sx = 0, sy = 0;
                 if (lane == 0) {
-                    sx = atomicAdd(&st->x, 0u);
-                    sy = atomicAdd(&st->y, 0u);
+                    __threadfence();
+                    last = (atomicAdd(&st->z, 1u) == chunks - 1u) ? 1u : 0u;
+                    if (last) {
+                        __threadfence();
+                        sx = atomicAdd(&st->x, 0u);
+                        sy = atomicAdd(&st->y, 0u);
+                    }
                 }
-                sx = __shfl_sync(kFull, sx, 0);
-                sy = __shfl_sync(kFull, sy, 0);
-                uniform = query ? (sy == 0u && sx != kNone) : (sx == sy);
-                wv = sx;
-                decided = true;
+                decided = __shfl_sync(kFull, last, 0) != 0u;
+                wv = __shfl_sync(kFull, sx, 0);
+                uniform = wv == __shfl_sync(kFull, sy, 0);
             }
         }
 
@@ -765,26 +844,31 @@ cudaError_t launch_init(uint2 *olt0, uint4 *rst0, DevCounters *ctr, uint32_t n, 
     return cudaGetLastError();
 }
 
-template <bool COUNT, bool BATCH>
+template <bool COUNT, bool BATCH, int NS>
 static void level_launch(const LevelArgs &a, int sms, cudaStream_t s)
 {
-    const size_t smem = (size_t)(256 / 32) * kWarpStage * sizeof(uint32_t);
-    const int grid = persistent_grid(level_kernel<COUNT, BATCH>, 256, smem, sms);
-    level_kernel<COUNT, BATCH><<<grid, 256, smem, s>>>(a);
+    const size_t smem = a.exact_last ? (size_t)(256 / 32) * kWarpStage * sizeof(uint32_t) : 0u;
+    // no more CTAs than the level can have items for
+    const unsigned long long most = ((unsigned long long)a.bound * a.chunks + 7u) / 8u;
+    int grid = persistent_grid(level_kernel<COUNT, BATCH, NS>, 256, smem, sms);
+    if (most < (unsigned long long)grid)
+        grid = most ? (int)most : 1;
+    level_kernel<COUNT, BATCH, NS><<<grid, 256, smem, s>>>(a);
 }
 
 cudaError_t launch_level(const LevelArgs &a, bool count, bool batch, int sms, cudaStream_t s)
 {
+    const bool two = a.chunks > 1u || a.side > kLevelSide1;
     if (batch) {
         if (count)
-            level_launch<true, true>(a, sms, s);
+            two ? level_launch<true, true, 2>(a, sms, s) : level_launch<true, true, 1>(a, sms, s);
         else
-            level_launch<false, true>(a, sms, s);
+            two ? level_launch<false, true, 2>(a, sms, s) : level_launch<false, true, 1>(a, sms, s);
     } else {
         if (count)
-            level_launch<true, false>(a, sms, s);
+            two ? level_launch<true, false, 2>(a, sms, s) : level_launch<true, false, 1>(a, sms, s);
         else
-            level_launch<false, false>(a, sms, s);
+            two ? level_launch<false, false, 2>(a, sms, s) : level_launch<false, false, 1>(a, sms, s);
     }
     return cudaGetLastError();
 }
@@ -812,7 +896,11 @@ template <bool COUNT, bool BATCH>
 static void refill_launch(const LeafArgs &a, int sms, cudaStream_t s)
 {
     const int threads = kRefillWarps * 32;
-    const int grid = persistent_grid(leaf_refill_kernel<COUNT, BATCH>, threads, 0, sms);
+    // no more CTAs than the leaves can have pre-passes for
+    const unsigned long long most = a.bound * a.side * a.side / (64u * kRefillWarps) + 1u;
+    int grid = persistent_grid(leaf_refill_kernel<COUNT, BATCH>, threads, 0, sms);
+    if (most < (unsigned long long)grid)
+        grid = (int)most;
     leaf_refill_kernel<COUNT, BATCH><<<grid, threads, 0, s>>>(a);
 }
 

@@ -219,10 +219,10 @@ extern "C" ask_status ask_render_noalloc(const ask_window *window, uint32_t n, u
         a.olt_cap = kNoAllocRegions;
         a.in_cap = kNoAllocRegions;  // the tables fill from both ends of the whole array
         a.out_cap = kNoAllocRegions;
+        a.bound = plan.max_regions[i];
         // one warp per region and fills in place: no per-region query state
         // or fill list, so the fixed scratch stays at three tables
         a.chunks = 1u;
-        a.chunk_px = kChunkPx;
         a.next_chunks = 1u;
         a.rst_in = nullptr;
         a.rst_out = nullptr;
@@ -243,6 +243,7 @@ extern "C" ask_status ask_render_noalloc(const ask_window *window, uint32_t n, u
     la.side = plan.side[L - 1];
     la.leaves = sc->leaves;
     la.leaf_cap = kNoAllocRegions;
+    la.bound = plan.max_regions[L - 1];
     la.skip_perimeter = 0u;
     la.fills = nullptr;
     la.fill_cap = 0u;

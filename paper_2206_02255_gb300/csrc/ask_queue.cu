@@ -236,30 +236,10 @@ __device__ __forceinline__ void process_item(const QueueArgs &q, uint32_t t, uin
     uint32_t wv = 0;
     if (C <= 1u) {
         decided = true;
-        uniform = warp_perimeter_uniform<kQueryRoundBatch, kBatchShortWhole>(f.pm, f.max_dwell, g, lane, &wv, it);
+        uniform = warp_perimeter_uniform<kQueryRound, 1>(f.pm, f.max_dwell, g, lane, &wv, it);
     } else {
         uint4 *st = q.rst + aux;
-        const uint32_t CP = max(q.chunk_px, ceil_div_u32(P, C));
-        const uint32_t k0 = min(P, c * CP), k1 = min(P, k0 + CP);
-        if (k0 < k1)
-            chunk_query<true>(f, g, k0, k1, st, lane, it);
-        // the warp that finishes the region's last chunk decides
-        uint32_t last = 0;
-        if (lane == 0)
-            last = (atomic_add_acq_rel(&st->z, 1u) == C - 1u) ? 1u : 0u;
-        last = __shfl_sync(kFull, last, 0);
-        if (last) {
-            uint32_t sx = 0, sy = 0;
-            if (lane == 0) {
-                sx = atomicAdd(&st->x, 0u);
-                sy = atomicAdd(&st->y, 0u);
-            }
-            sx = __shfl_sync(kFull, sx, 0);
-            sy = __shfl_sync(kFull, sy, 0);
-            uniform = (sy == 0u && sx != kNone);
-            wv = sx;
-            decided = true;
-        }
+        decided = chunk_decides(chunk_query<true, 1>(f, g, P, c, C, st, lane, it), st, C, lane, uniform, wv);
     }
     if (COUNT) {
         it = warp_sum_u64(it);
@@ -563,6 +543,7 @@ cudaError_t launch_queue(const QueueArgs &q, uint32_t nframes, bool count, int s
     a.side = 0;
     a.leaves = q.leaves;
     a.leaf_cap = q.leaf_cap;
+    a.bound = 0;
     a.skip_perimeter = 0;
     a.fills = nullptr;
     a.fill_cap = 0;

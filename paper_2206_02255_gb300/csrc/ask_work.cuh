@@ -83,111 +83,83 @@ __device__ __forceinline__ FView view_frame(const FrameDesc *frames, uint32_t f,
     return v;
 }
 
-// Rounds between issuing a state load and using it, for one frame.  A
-// batch keeps enough warps resident to hide the load, and there a late
-// stop costs more than the wait, so it uses the value one round later.
-constexpr uint32_t kPollLag = 8;
 // Chunked queries of regions with longer perimeters skip the short first
-// rounds of query_step (at n = 16384 they slowed levels 0 and 1, whose
-// regions of side 1024 and 256 are seldom uniform outside the set, and sped
-// up level 2, side 64).
+// rounds of query_group: such regions are seldom uniform outside the set
+// (without short rounds for any chunk level 2 at n = 16384, side 64, took 229
+// us against 211, with them for every chunk level 0 the same as without).
 constexpr uint32_t kShortRoundsMaxPerimeter = 512;
 
-// One chunk [k0, k1) of a large region's perimeter, queried by one warp.  The
-// region's state st: x = common dwell found so far (kNone: none yet),
-// y = 1 once two dwells are known to differ, z = chunks finished.  Chunks of
-// the same region run on other warps at the same time and stop as soon as
-// one of them has set y.
-template <bool BATCH>
-__device__ __forceinline__ void chunk_query(const FView &a, const Region &g, uint32_t k0,
-                                            uint32_t k1, uint4 *st, uint32_t lane,
-                                            unsigned long long &it)
+// Chunk c of the `chunks` of a large region's perimeter (P pixels), queried
+// by one warp: the pixels c, c + chunks, c + 2 chunks, ..., so that every
+// chunk, and every group of 32 * NS in it, is spread over the whole perimeter.  The
+// region's state st: x = common dwell found so far (kNone: none yet), y = 1
+// once two dwells are known to differ, z = chunks finished without.  Chunks
+// of the same region run on other warps at the same time and stop as soon as
+// one of them has set y.  Returns whether this chunk found the difference
+// first (GROUP_DIFFER: the caller decides the region), found none
+// (GROUP_SAME), or stopped because another did (GROUP_STOP).
+template <bool BATCH, int NS>
+__device__ __forceinline__ uint32_t chunk_query(const FView &a, const Region &g, uint32_t P, uint32_t c,
+                                                uint32_t chunks, uint4 *st, uint32_t lane,
+                                                unsigned long long &it)
 {
     const volatile uint32_t *ps = reinterpret_cast<const volatile uint32_t *>(st);
-    for (uint32_t base = k0; base < k1; base += 32u) {
-        // the state load is issued first; the group's set-up hides its latency
-        uint32_t sx = 0, sy = 0;
+    const uint32_t n = P > c ? (P - c + chunks - 1u) / chunks : 0u;
+    const uint32_t rnd = P <= kShortRoundsMaxPerimeter ? 0u : 3u;
+    constexpr uint32_t K = kQueryRound, lag = BATCH ? 1u : kPollLag;
+    for (uint32_t base = 0; base < n; base += 32u * NS) {
+        uint32_t sx = 0, sy = 0, vmin = 0, vmax = 0;
         if (lane == 0) {
             sx = ps[0];
             sy = ps[1];
         }
-        const uint32_t k = base + lane;
-        const bool active = k < k1;
-        const unsigned amask = __ballot_sync(kFull, active);
-        uint32_t px = g.x0, py = g.y0;
-        if (active)
-            perimeter_pixel(g, k, px, py);
-        Orbit o = orbit_start(pixel_c(a.pm, px, py));
-        uint32_t stt = active ? ORBIT_RUN : ORBIT_DONE;
-        bool differ = false, stop = false;
-        uint2 v = make_uint2(__shfl_sync(kFull, sx, 0), __shfl_sync(kFull, sy, 0));
-        if (v.y)
-            return;
-        // A state load is issued every kPollLag rounds (every round in a
-        // batch) and consumed that many rounds later, so its L2 latency
-        // hides behind the updates of those rounds; a stale value is
-        // harmless (the common dwell is set once, the flag only rises).
-        // short first rounds for small regions only: large ones are mostly
-        // inside the set or on its boundary, rarely uniform outside it
-        uint32_t nx = v.x, ny = v.y, lag = 0;
-        constexpr bool kShort = !BATCH || kBatchShortChunks;
-        uint32_t rnd = (kShort && perimeter_size(g.w, g.h) <= kShortRoundsMaxPerimeter) ? 0u : 3u;
-        for (;; ++rnd) {
-            if (lag == 0 && lane == 0) {
-                nx = ps[0];
-                ny = ps[1];
-            }
-            const uint32_t limit = (v.x != kNone) ? min(a.max_dwell, v.x + 1u) : a.max_dwell;
-            if (kShort)
-                query_step<kQueryRoundLarge>(o, stt, limit, rnd);
-            else if (stt == ORBIT_RUN)
-                stt = orbit_step<kQueryRoundLarge>(o, limit);
-            const unsigned dm = __ballot_sync(kFull, stt != ORBIT_RUN) & amask;
-            if (dm == amask)
-                break;
-            if (dm) {
-                differ = true;
-                break;
-            }
-            if (++lag == (BATCH ? 1u : kPollLag)) {
-                lag = 0;
-                v.x = __shfl_sync(kFull, nx, 0);
-                v.y = __shfl_sync(kFull, ny, 0);
-                if (v.y) {
-                    stop = true;
-                    break;
-                }
-            }
+        if (__shfl_sync(kFull, sy, 0))
+            return GROUP_STOP;
+        sx = __shfl_sync(kFull, sx, 0);
+        const uint32_t r = spread_group<K, NS>(a.pm, a.max_dwell, g, c, chunks, base, P, rnd, sx, ps, lag,
+                                               lane, vmin, vmax, it);
+        if (r == GROUP_STOP)
+            return r;
+        bool differ = (r == GROUP_DIFFER);
+        if (!differ) {
+            uint32_t old = kNone;
+            if (vmin == vmax && lane == 0)
+                old = atomicCAS(&st->x, kNone, vmin);
+            old = __shfl_sync(kFull, old, 0);
+            differ = vmin != vmax || (old != kNone && old != vmin);
         }
-        // every orbit finished in round rnd (else they would differ)
-        if (!stop && !differ && stt == ORBIT_PEND) {
-            if (kShort)
-                query_resolve<kQueryRoundLarge>(o, rnd);
-            else
-                orbit_resolve<kQueryRoundLarge>(o);
-        }
-        if (active)
-            it += o.d;
-        if (stop)
-            return;
         if (differ) {
+            uint32_t first = 0;
             if (lane == 0)
-                atomicExch(&st->y, 1u);
-            return;
+                first = atomicExch(&st->y, 1u) == 0u ? 1u : 0u;
+            return __shfl_sync(kFull, first, 0) ? GROUP_DIFFER : GROUP_STOP;
         }
-        const uint32_t vmin = __reduce_min_sync(kFull, active ? o.d : kNone);
-        const uint32_t vmax = __reduce_max_sync(kFull, active ? o.d : 0u);
-        if (lane == 0) {
-            if (vmin != vmax) {
-                atomicExch(&st->y, 1u);
-            } else {
-                const uint32_t old = atomicCAS(&st->x, kNone, vmin);
-                if (old != kNone && old != vmin)
-                    atomicExch(&st->y, 1u);
-            }
-        }
-        __syncwarp();
     }
+    return GROUP_SAME;
+}
+
+// After chunk_query: whether this warp decides the region, and how.  The warp
+// that found the difference decides at once; with none, the warp that
+// finishes the last of the chunks does (a chunk that found a difference never
+// counts as finished, so exactly one warp decides).
+__device__ __forceinline__ bool chunk_decides(uint32_t r, uint4 *st, uint32_t chunks, uint32_t lane,
+                                              bool &uniform, uint32_t &wv)
+{
+    uniform = false;
+    if (r != GROUP_SAME)
+        return r == GROUP_DIFFER;
+    uint32_t last = 0, x = 0;
+    if (lane == 0) {
+        __threadfence();
+        last = (atomicAdd(&st->z, 1u) == chunks - 1u) ? 1u : 0u;
+        if (last) {
+            __threadfence();
+            x = atomicAdd(&st->x, 0u);
+        }
+    }
+    wv = __shfl_sync(kFull, x, 0);
+    uniform = true;
+    return __shfl_sync(kFull, last, 0) != 0u;
 }
 
 // ---------------------------------------------------------------------------
