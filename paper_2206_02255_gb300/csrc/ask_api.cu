@@ -1642,6 +1642,7 @@ ask_status render64_impl(ask_ctx *ctx, ask_method method, const ask_window64 *wi
     la.max_dwell = max_dwell;
     la.leaves = ctx->leaves;
     la.leaf_cap = (uint32_t)ctx->leaf_cap;
+    la.side = plan.side[L - 1];
     la.ctr = ctx->ctr;
     if ((e = launch_leaf64(la, count, ff, ctx->dev.sms, s)) != cudaSuccess)
         return cuda_err(ctx, e, "double-precision leaf kernel");

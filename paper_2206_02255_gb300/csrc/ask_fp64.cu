@@ -24,12 +24,14 @@
 //    lockstep rounds, so the query stops as soon as one orbit has finished
 //    while another still runs; uniform regions are filled in place;
 //  * leaf kernel: persistent; a lane whose orbit ends takes the next pixel
-//    of its warp's current leaf (then of the next leaf) at once; an orbit
+//    of its warp's current band of a leaf (then of the next band) at once; an orbit
 //    that escapes inside an unchecked block is parked in shared memory and
 //    32 parked orbits are resolved together, so no lane replays alone.
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "ask_device.cuh"
 #include "ask_fp64.h"
@@ -39,16 +41,21 @@ namespace ask {
 namespace {
 
 constexpr unsigned kAll = 0xffffffffu;
-// Updates per unchecked block of the exhaustive kernel's dwell loop, and per
-// lockstep round of the perimeter queries and of the leaf kernel's orbits.
+// Updates per unchecked block of the exhaustive kernel's dwell loop.
 constexpr uint32_t kBlock64 = 16;
-constexpr uint32_t kRound64 = 8;
 // |c|^2 bounds below which escape is absorbing (see the policies' absorbing()).
 constexpr double kAbsorbR2_F64 = 3.999;
 constexpr float kAbsorbR2_FF = 3.999f;
 // Leaf kernel: warps per CTA and parked orbits per warp (fewer than 32 wait
 // between resolves, and one round parks at most 32 more).
 constexpr uint32_t kLeaf64Warps = 4;
+// Level kernel: warps per CTA.
+constexpr uint32_t kLevel64Warps = 4;
+// Leaves are handed out as 1 << shift row bands each, cut until every warp
+// gets kLeaf64Items or a band of a full leaf would hold fewer than 32 pixels:
+// with whole leaves as items, 962 leaves of 32 x 32 went to 962 warps on a part
+// of the SMs (20.5 ms against 9.0).
+constexpr uint32_t kLeaf64Items = 16;
 constexpr uint32_t kPark64 = 64;
 
 __device__ __forceinline__ double2 pixel_c64(const PixelMap64 &pm, uint32_t px, uint32_t py)
@@ -60,6 +67,18 @@ __device__ __forceinline__ double2 pixel_c64(const PixelMap64 &pm, uint32_t px, 
 // Binary64: one update z <- z^2 + c, each operation rounded once to double.
 struct ArithF64 {
     using T = double;
+    // Updates per unchecked block of the queries' and the leaf kernel's rounds
+    // (the test after each is 2 instructions of the FP64 pipe beside the
+    // block's 64: 8 updates took 9.36 ms on the map below, 16 9.11).
+    static constexpr uint32_t kRound = 16;
+    // CTAs an SM.  A warp instruction holds the SM's FP64 pipe for 16 cycles
+    // however few lanes take part, and 2 warps a scheduler keep it busy, so
+    // more warps only leave more half-empty ones at the end: n = 1024 in
+    // seahorse valley (2^-30 wide, cap 4096, g=32 r=4 B=16), leaf kernel 8.95 /
+    // 9.04 / 9.34 / 9.43 ms with 2 / 4 / 8 / 16 CTAs of 4 warps, level kernel
+    // 0.79 / 0.96 / 1.32 with 2 / 3 / 10.
+    static constexpr int kLeafCtas = 2;
+    static constexpr int kLevelCtas = 2;
     static __device__ __forceinline__ T from_double(double v) { return v; }
     static __device__ __forceinline__ void update(T &x, T &y, T cr, T ci)
     {
@@ -71,7 +90,10 @@ struct ArithF64 {
     }
     static __device__ __forceinline__ bool bounded(T x, T y)
     {
-        return __fma_rn(x, x, __dmul_rn(y, y)) < 4.0;
+        // m < 4 read off the high word (4.0 is 0x40100000'00000000, m is never
+        // negative; inf and NaN of either sign compare above), which keeps
+        // the comparison off the FP64 pipe
+        return (uint32_t)__double2hiint(__fma_rn(x, x, __dmul_rn(y, y))) < 0x40100000u;
     }
     // The single-precision argument carries over with a wider margin: for
     // |c|^2 < 3.999, a rounded |z_j|^2 >= 4 means the exact |z_j|^2 exceeds
@@ -100,6 +122,13 @@ struct ArithF64 {
 // lo = (float)(c - hi).  About 60 FP32 instructions per update.
 struct ArithFF {
     using T = float2;
+    // (n = 3000 on the antenna, 2^-20 wide, cap 2048, g=64 r=4 B=8: 7.77 ms
+    // with 8 updates a round, 7.25 with 16, 8.70 with 32 fully unrolled)
+    static constexpr uint32_t kRound = 16;
+    // CTAs of 4 warps an SM: leaf kernel 5.93 / 5.58 / 5.51 / 5.57 ms with 4 /
+    // 6 / 8 / 16; level 0 0.58 / 0.49 with 8 / 4.
+    static constexpr int kLeafCtas = 8;
+    static constexpr int kLevelCtas = 4;
     static __device__ __forceinline__ float2 fast_two_sum(float a, float b)
     {
         const float s = __fadd_rn(a, b);
@@ -267,8 +296,8 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v)
     return v;
 }
 
-// One warp queries the whole perimeter of g (Q of Sec. 4.2.1): 32 perimeter
-// pixels at a time, their orbits in lockstep rounds.  An orbit still running
+// One warp queries the whole perimeter of g (Q of Sec. 4.2.1): 32 pixels
+// spread over it at a time, their orbits in lockstep rounds.  An orbit still running
 // after a round has made more updates than any that finished in it, so one
 // finished and one running orbit prove the perimeter non-uniform.  Once a
 // group ends with a common dwell w, later groups stop at w + 1 updates.
@@ -279,10 +308,11 @@ __device__ __forceinline__ bool warp_uniform_w(const PixelMap64 &pm, uint32_t ma
                                                unsigned long long &it)
 {
     const uint32_t P = perimeter_size(g.w, g.h);
+    const uint32_t groups = (P + 31u) / 32u;
     bool have = false;
     uint32_t w = 0;
-    for (uint32_t base = 0; base < P; base += 32u) {
-        const uint32_t k = base + lane;
+    for (uint32_t j = 0; j < groups; ++j) {
+        const uint32_t k = j + lane * groups;
         const bool active = k < P;
         const unsigned amask = __ballot_sync(kAll, active);
         uint32_t px = g.x0, py = g.y0;
@@ -294,7 +324,7 @@ __device__ __forceinline__ bool warp_uniform_w(const PixelMap64 &pm, uint32_t ma
         bool differ = false;
         for (;;) {
             if (stt == ORBIT_RUN)
-                stt = orbit_w_step<A, kRound64>(o, limit);
+                stt = orbit_w_step<A, A::kRound>(o, limit);
             const unsigned dm = __ballot_sync(kAll, stt != ORBIT_RUN) & amask;
             if (dm == amask)
                 break;
@@ -304,7 +334,7 @@ __device__ __forceinline__ bool warp_uniform_w(const PixelMap64 &pm, uint32_t ma
             }
         }
         if (!differ && stt == ORBIT_PEND)
-            orbit_w_resolve<A, kRound64>(o);
+            orbit_w_resolve<A, A::kRound>(o);
         if (active)
             it += o.d;
         if (differ)
@@ -350,7 +380,7 @@ __global__ void __launch_bounds__(1024) exhaustive64_kernel(uint32_t *__restrict
 // Sec. 5.3.1) or leaf.
 // ---------------------------------------------------------------------------
 template <class A, bool COUNT>
-__global__ void __launch_bounds__(256) level64_kernel(Level64Args a)
+__global__ void __launch_bounds__(kLevel64Warps * 32) level64_kernel(Level64Args a)
 {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t total = min(a.ctr->count[a.level], a.olt_cap);
@@ -429,12 +459,22 @@ __device__ __forceinline__ void resolve_parked_w(const Leaf64Args &a, ParkW<A> &
     q.d = pk.d[wid][e];
     q.fast = true;
     const uint32_t pix = pk.pix[wid][e];
-    orbit_w_resolve<A, kRound64>(q);
+    orbit_w_resolve<A, A::kRound>(q);
     a.map[(size_t)(pix >> 16) * a.n + (pix & 0xffffu)] = q.d;
     if (COUNT) {
         it += q.d;
         ++npx;
     }
+}
+
+__device__ __forceinline__ uint32_t leaf_item_shift64(uint32_t leaves, uint32_t side, uint32_t warps)
+{
+    const unsigned long long px = (unsigned long long)side * side;
+    uint32_t shift = 0;
+    while (((unsigned long long)leaves << shift) < (unsigned long long)kLeaf64Items * warps &&
+           (px >> (shift + 1u)) >= 32u && (2u << shift) <= side)
+        ++shift;
+    return shift;
 }
 
 template <class A, bool COUNT>
@@ -444,6 +484,7 @@ __global__ void __launch_bounds__(kLeaf64Warps * 32) leaf64_kernel(Leaf64Args a)
     const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
     const uint32_t nleaves = min(a.ctr->leaf_count, a.leaf_cap);
+    const uint32_t shift = leaf_item_shift64(nleaves, a.side, gridDim.x * kLeaf64Warps);
     // warp-uniform: the leaf being handed out and how many of its pixels are
     Region cur;
     cur.x0 = cur.y0 = 0;
@@ -464,11 +505,19 @@ __global__ void __launch_bounds__(kLeaf64Warps * 32) leaf64_kernel(Leaf64Args a)
                 if (lane == 0u)
                     li = atomicAdd(&a.ctr->leaf_work, 1u);
                 li = __shfl_sync(kAll, li, 0);
-                if (li >= nleaves) {
+                if ((li >> shift) >= nleaves) {
                     exhausted = true;
                     break;
                 }
-                cur = unpack_region(a.leaves[li]);
+                cur = unpack_region(a.leaves[li >> shift]);
+                // rows [r0, r1) of the leaf
+                const uint32_t band = li & ((1u << shift) - 1u);
+                const uint32_t r0 = (uint32_t)(((unsigned long long)cur.h * band) >> shift);
+                const uint32_t r1 = (uint32_t)(((unsigned long long)cur.h * (band + 1u)) >> shift);
+                if (r0 == r1)
+                    continue;
+                cur.y0 += r0;
+                cur.h = r1 - r0;
                 next = 0;
                 npix = (unsigned long long)cur.w * cur.h;
                 have = true;
@@ -493,7 +542,7 @@ __global__ void __launch_bounds__(kLeaf64Warps * 32) leaf64_kernel(Leaf64Args a)
             break;
         uint32_t st = ORBIT_RUN;
         if (busy) {
-            st = orbit_w_step<A, kRound64>(o, a.max_dwell);
+            st = orbit_w_step<A, A::kRound>(o, a.max_dwell);
             if (st == ORBIT_DONE) {
                 a.map[(size_t)(pix >> 16) * a.n + (pix & 0xffffu)] = o.d;
                 if (COUNT) {
@@ -577,7 +626,9 @@ cudaError_t launch_exhaustive64(uint32_t *map, uint32_t n, PixelMap64 pm, uint32
 template <class A, bool COUNT>
 static void level_w_launch(const Level64Args &a, int sms, cudaStream_t s)
 {
-    level64_kernel<A, COUNT><<<resident_grid(level64_kernel<A, COUNT>, 256, sms), 256, 0, s>>>(a);
+    const int threads = (int)kLevel64Warps * 32;
+    const int grid = std::min(resident_grid(level64_kernel<A, COUNT>, threads, sms), A::kLevelCtas * sms);
+    level64_kernel<A, COUNT><<<grid, threads, 0, s>>>(a);
 }
 
 cudaError_t launch_level64(const Level64Args &a, bool count, bool ff, int sms, cudaStream_t s)
@@ -593,7 +644,8 @@ template <class A, bool COUNT>
 static void leaf_w_launch(const Leaf64Args &a, int sms, cudaStream_t s)
 {
     const int threads = (int)kLeaf64Warps * 32;
-    leaf64_kernel<A, COUNT><<<resident_grid(leaf64_kernel<A, COUNT>, threads, sms), threads, 0, s>>>(a);
+    const int grid = std::min(resident_grid(leaf64_kernel<A, COUNT>, threads, sms), A::kLeafCtas * sms);
+    leaf64_kernel<A, COUNT><<<grid, threads, 0, s>>>(a);
 }
 
 cudaError_t launch_leaf64(const Leaf64Args &a, bool count, bool ff, int sms, cudaStream_t s)

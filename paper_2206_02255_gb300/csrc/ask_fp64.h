@@ -41,6 +41,7 @@ struct Leaf64Args {
     uint32_t max_dwell;
     const uint2 *leaves;
     uint32_t leaf_cap;
+    uint32_t side;        // nominal side of the leaf regions
     DevCounters *ctr;
 };
 
