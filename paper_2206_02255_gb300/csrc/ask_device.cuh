@@ -10,8 +10,11 @@
 
 namespace ask {
 
-// Updates per unchecked block in the dwell loops (see dwell()).
-constexpr int kUnroll = 16;
+// Updates per unchecked block of the dwell loops: the first and the others of
+// the loop with proofs, and those of the plain loop (see dwell()).
+constexpr int kFirstBlock = 16;
+constexpr int kUnroll = 32;
+constexpr int kPlainBlock = 16;
 
 // |c|^2 bound below which escape is absorbing in float arithmetic (see dwell()).
 constexpr float kAbsorbR2 = 3.999f;
@@ -106,40 +109,6 @@ __device__ __forceinline__ bool escape_absorbing(float cr, float ci)
     return __fmaf_rn(cr, cr, __fmul_rn(ci, ci)) < kAbsorbR2;
 }
 
-// Dwell of c (paper Sec. 6): the number of updates z <- z^2 + c, from z = 0,
-// made while |z|^2 < 4, at most max_dwell.
-//
-// Where escape is absorbing, updates run in blocks of kUnroll with a single
-// test on the block's last state: 3 FFMA + 1 FADD per update, the test
-// amortised over the block.  A block whose last state fails the test is
-// rolled back and replayed one tested update at a time, so the count is
-// exactly the stepwise one.  Other points, and the tail below max_dwell, take
-// the tested loop.
-__device__ __forceinline__ uint32_t dwell(float cr, float ci, uint32_t max_dwell)
-{
-    float x = 0.0f, y = 0.0f;
-    uint32_t d = 0;
-    if (escape_absorbing(cr, ci)) {
-        while (max_dwell - d >= (uint32_t)kUnroll) {
-            const float sx = x, sy = y;
-#pragma unroll
-            for (int k = 0; k < kUnroll; ++k)
-                z_update(x, y, cr, ci);
-            if (!z_bounded(x, y)) {
-                x = sx;
-                y = sy;
-                break;
-            }
-            d += (uint32_t)kUnroll;
-        }
-    }
-    while (d < max_dwell && z_bounded(x, y)) {
-        z_update(x, y, cr, ci);
-        ++d;
-    }
-    return d;
-}
-
 __device__ __forceinline__ float sqrt_approx(float v)
 {
     float r;
@@ -215,6 +184,147 @@ __device__ __forceinline__ void capture_disc(float cr, float ci, float x, float 
     const float r1 = r * (A + r) + q1;
     if (r > 0.0f && r1 * (B + r1) + q2 <= 0.9999f * r && 0.5f * A + r < 1.9f && 0.5f * B + r1 < 1.9f)
         r2 = 0.9999f * r * r;
+}
+
+// Whether c can have a capture disc at all: it lies in the main cardioid or in
+// the period-2 disc (up to rounding; a filter that saves the others the work:
+// n = 3001 at zoom 60 408 -> 393 us, n = 1999 at zoom 300 311 -> 284 us).
+__device__ __forceinline__ bool may_capture(float cr, float ci)
+{
+    const float u = cr - 0.25f, i2 = ci * ci, q = __fmaf_rn(u, u, i2), v = cr + 1.0f;
+    return q * (q + u) < 0.25f * i2 || __fmaf_rn(v, v, i2) < 0.0625f;
+}
+
+// Whether the orbit of c, at state (x, y), is in its capture disc.
+__device__ __forceinline__ bool captured(float cr, float ci, float x, float y)
+{
+    float ax, ay, r2;
+    capture_disc(cr, ci, x, y, ax, ay, r2);
+    const float ux = x - ax, uy = y - ay;
+    return __fmaf_rn(ux, ux, __fmul_rn(uy, uy)) < r2;
+}
+
+// Dwell of an orbit whose state (x, y) at count d passed the test and whose
+// state K updates later failed, where escape is absorbing: halving the gap
+// finds the first failing state (K - 1 updates, log2(K) tests).
+template <uint32_t K>
+__device__ __forceinline__ uint32_t dwell_in_block(float x, float y, float cr, float ci, uint32_t d)
+{
+#pragma unroll
+    for (uint32_t h = K / 2u; h >= 1u; h >>= 1) {
+        float tx = x, ty = y;
+#pragma unroll
+        for (uint32_t k = 0; k < h; ++k)
+            z_update(tx, ty, cr, ci);
+        if (z_bounded(tx, ty)) {
+            x = tx;
+            y = ty;
+            d += h;
+        }
+    }
+    return d + 1u;
+}
+
+// Dwell of c (paper Sec. 6): the number of updates z <- z^2 + c, from z = 0,
+// made while |z|^2 < 4, at most max_dwell.
+//
+// Where escape is absorbing, updates run in blocks with a single test on the
+// block's last state: 3 FFMA + 1 FADD per update, the test amortised over the
+// block; a block whose last state fails the test holds the dwell, which is
+// found behind the loop, so that the lanes of a warp do it together, and is
+// exactly the stepwise count.  Other points, and the tail below max_dwell, take
+// the tested loop.
+//
+// Two loops do this.  A warp with a point that may have a capture disc takes
+// blocks of kFirstBlock and then kUnroll, and every two of them ends the orbits
+// that would stay for ever: those that repeat a saved state and, at doubling
+// counts, when the state is saved anew, those that have entered their disc.  A
+// warp with none takes the plain loop (blocks of kPlainBlock, replayed by
+// tested updates): the proofs would cost a zoom outside the two largest
+// components 3-6%.  The exhaustive kernel at n = 16384, cap 2048, over the whole
+// set: 28.8 ms with every orbit of the set run to the cap, 6.28 this way; n =
+// 4096 1.86 -> 0.46 ms; n = 2048 at zoom 400, cap 1024: 0.259 -> 0.258.
+__device__ __forceinline__ uint32_t dwell(float cr, float ci, uint32_t max_dwell)
+{
+    float x = 0.0f, y = 0.0f;
+    uint32_t d = 0;
+    if (escape_absorbing(cr, ci)) {
+        const bool may = may_capture(cr, ci);
+        if (__any_sync(__activemask(), may)) {  // (either loop gives the same dwell)
+            float bx = 0.0f, by = 0.0f, tx = 0.0f, ty = 0.0f;
+            uint32_t age = 0;
+            bool esc = false, in = false;
+            if (max_dwell >= (uint32_t)kFirstBlock) {
+#pragma unroll
+                for (int k = 0; k < kFirstBlock; ++k)
+                    z_update(tx, ty, cr, ci);
+                if (!z_bounded(tx, ty))
+                    return dwell_in_block<kFirstBlock>(0.0f, 0.0f, cr, ci, 0u);
+                x = bx = tx;
+                y = by = ty;
+                d = (uint32_t)kFirstBlock;
+            }
+            while (max_dwell - d >= (uint32_t)kUnroll) {
+                tx = x;
+                ty = y;
+#pragma unroll
+                for (int k = 0; k < kUnroll; ++k)
+                    z_update(tx, ty, cr, ci);
+                esc = !z_bounded(tx, ty);
+                if (esc)
+                    break;
+                x = tx;
+                y = ty;
+                d += (uint32_t)kUnroll;
+                age += (uint32_t)kUnroll;
+                if (age % (2u * kUnroll) == 0u) {
+                    in = x == bx && y == by;
+                    if (!in && (age & (age - 1u)) == 0u) {
+                        in = may && captured(cr, ci, x, y);
+                        bx = x;
+                        by = y;
+                    }
+                    if (in)
+                        break;
+                }
+            }
+            if (in)
+                return max_dwell;
+            if (esc)
+                return dwell_in_block<kUnroll>(x, y, cr, ci, d);
+        } else {
+            while (max_dwell - d >= (uint32_t)kPlainBlock) {
+                const float sx = x, sy = y;
+#pragma unroll
+                for (int k = 0; k < kPlainBlock; ++k)
+                    z_update(x, y, cr, ci);
+                if (!z_bounded(x, y)) {
+                    x = sx;
+                    y = sy;
+                    break;
+                }
+                d += (uint32_t)kPlainBlock;
+            }
+        }
+    }
+    while (d < max_dwell && z_bounded(x, y)) {
+        z_update(x, y, cr, ci);
+        ++d;
+    }
+    return d;
+}
+
+// The same by tested updates alone (perimeter groups with points of |c| near
+// 2; out of line, off the queries' way).
+static __device__ __noinline__ uint32_t dwell_tested(float cr, float ci, uint32_t limit)
+{
+    float x = 0.0f, y = 0.0f;
+    uint32_t d = 0;
+    while (d < limit && z_bounded(x, y)) {
+        z_update(x, y, cr, ci);
+        ++d;
+    }
+    return d;
 }
 
 // Resumable orbit of one point, for perimeter queries that stop early.
@@ -554,7 +664,7 @@ __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max
 {
     float x[NS], y[NS], cr[NS], ci[NS];
     float bx[NS], by[NS], ax[NS], ay[NS], r2[NS];
-    bool run[NS], pend[NS];
+    bool run[NS], pend[NS], may[NS];
     bool plain = false;
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
@@ -566,6 +676,7 @@ __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max
         r2[i] = -1.0f;
         run[i] = active[i];
         pend[i] = false;
+        may[i] = may_capture(c.x, c.y);
         d[i] = 0;
         plain = plain || (active[i] && !escape_absorbing(c.x, c.y));
     }
@@ -575,7 +686,7 @@ __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max
 #pragma unroll
         for (int i = 0; i < NS; ++i)
             if (active[i])
-                d[i] = dwell(cr[i], ci[i], limit);
+                d[i] = dwell_tested(cr[i], ci[i], limit);
         return GROUP_SAME;
     }
     uint32_t n = 0;  // updates made by the running orbits
@@ -607,7 +718,7 @@ __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max
             for (int i = 0; i < NS; ++i) {
                 bx[i] = x[i];
                 by[i] = y[i];
-                if (run[i])
+                if (run[i] && may[i])
                     capture_disc(cr[i], ci[i], x[i], y[i], ax[i], ay[i], r2[i]);
             }
         }
