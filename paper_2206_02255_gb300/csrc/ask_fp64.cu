@@ -35,6 +35,7 @@
 
 #include "ask_device.cuh"
 #include "ask_fp64.h"
+#include "ask_launch.cuh"
 
 namespace ask {
 
@@ -587,16 +588,6 @@ __global__ void __launch_bounds__(kLeaf64Warps * 32) leaf64_kernel(Leaf64Args a)
     }
 }
 
-template <typename K>
-int resident_grid(K kernel, int threads, int sms)
-{
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
-    return per_sm * sms;
-}
-
 }  // namespace
 
 cudaError_t launch_exhaustive64(uint32_t *map, uint32_t n, PixelMap64 pm, uint32_t max_dwell,
@@ -624,37 +615,35 @@ cudaError_t launch_exhaustive64(uint32_t *map, uint32_t n, PixelMap64 pm, uint32
 }
 
 template <class A, bool COUNT>
-static void level_w_launch(const Level64Args &a, int sms, cudaStream_t s)
+static cudaError_t level_w_launch(const Level64Args &a, int sms, cudaStream_t s)
 {
     const int threads = (int)kLevel64Warps * 32;
-    const int grid = std::min(resident_grid(level64_kernel<A, COUNT>, threads, sms), A::kLevelCtas * sms);
-    level64_kernel<A, COUNT><<<grid, threads, 0, s>>>(a);
+    static const int resident = std::min(resident_ctas(level64_kernel<A, COUNT>, threads, 0), A::kLevelCtas);
+    level64_kernel<A, COUNT><<<resident * sms, threads, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_level64(const Level64Args &a, bool count, bool ff, int sms, cudaStream_t s)
 {
     if (ff)
-        count ? level_w_launch<ArithFF, true>(a, sms, s) : level_w_launch<ArithFF, false>(a, sms, s);
-    else
-        count ? level_w_launch<ArithF64, true>(a, sms, s) : level_w_launch<ArithF64, false>(a, sms, s);
-    return cudaGetLastError();
+        return count ? level_w_launch<ArithFF, true>(a, sms, s) : level_w_launch<ArithFF, false>(a, sms, s);
+    return count ? level_w_launch<ArithF64, true>(a, sms, s) : level_w_launch<ArithF64, false>(a, sms, s);
 }
 
 template <class A, bool COUNT>
-static void leaf_w_launch(const Leaf64Args &a, int sms, cudaStream_t s)
+static cudaError_t leaf_w_launch(const Leaf64Args &a, int sms, cudaStream_t s)
 {
     const int threads = (int)kLeaf64Warps * 32;
-    const int grid = std::min(resident_grid(leaf64_kernel<A, COUNT>, threads, sms), A::kLeafCtas * sms);
-    leaf64_kernel<A, COUNT><<<grid, threads, 0, s>>>(a);
+    static const int resident = std::min(resident_ctas(leaf64_kernel<A, COUNT>, threads, 0), A::kLeafCtas);
+    leaf64_kernel<A, COUNT><<<resident * sms, threads, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_leaf64(const Leaf64Args &a, bool count, bool ff, int sms, cudaStream_t s)
 {
     if (ff)
-        count ? leaf_w_launch<ArithFF, true>(a, sms, s) : leaf_w_launch<ArithFF, false>(a, sms, s);
-    else
-        count ? leaf_w_launch<ArithF64, true>(a, sms, s) : leaf_w_launch<ArithF64, false>(a, sms, s);
-    return cudaGetLastError();
+        return count ? leaf_w_launch<ArithFF, true>(a, sms, s) : leaf_w_launch<ArithFF, false>(a, sms, s);
+    return count ? leaf_w_launch<ArithF64, true>(a, sms, s) : leaf_w_launch<ArithF64, false>(a, sms, s);
 }
 
 }  // namespace ask

@@ -44,6 +44,7 @@
 
 #include "ask_device.cuh"
 #include "ask_internal.h"
+#include "ask_launch.cuh"
 #include "ask_work.cuh"
 
 namespace ask {
@@ -112,6 +113,7 @@ __global__ void init_kernel(uint2 *__restrict__ olt0, uint4 *__restrict__ rst0, 
                             PixelMap pm, uint32_t order)
 {
     __shared__ uint32_t s_front, s_back;
+    chain_start();
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t total = axis0 * rows;
@@ -372,6 +374,7 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
     using R = Rec<BATCH>;
     using T = typename R::T;
     extern __shared__ uint32_t smem[];
+    chain_start();
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t *stage = smem + (threadIdx.x >> 5) * kWarpStage;
     const T *olt_in = static_cast<const T *>(a.olt_in);
@@ -701,6 +704,7 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocks) leaf_refi
 {
     __shared__ WarpLeaf<BATCH> shared[kRefillWarps];
     __shared__ uint3 extent;                           // front, leaves, item shift (LeafList)
+    chain_start();
     const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
         uint32_t front, total;
@@ -777,6 +781,7 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocks) leaf_refi
 __global__ void init_batch_kernel(uint4 *__restrict__ olt0, uint4 *__restrict__ rst0,
                                   DevCounters *ctr, const FrameDesc *frames, uint32_t total0)
 {
+    chain_start();
     const uint32_t f = blockIdx.x;
     if (f == 0) {
         uint32_t *w = reinterpret_cast<uint32_t *>(ctr);
@@ -796,16 +801,6 @@ __global__ void init_batch_kernel(uint4 *__restrict__ olt0, uint4 *__restrict__ 
         if (rst0 != nullptr)
             rst0[d.olt0_offset + k] = make_uint4(kNone, 0u, 0u, 0u);
     }
-}
-
-template <typename K>
-int persistent_grid(K kernel, int threads, size_t smem, int sms)
-{
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
-    return per_sm * sms;
 }
 
 }  // namespace
@@ -832,28 +827,30 @@ cudaError_t launch_init(uint2 *olt0, uint4 *rst0, DevCounters *ctr, uint32_t n, 
 {
     const uint32_t total = axis0 * rows;
     if (order != nullptr && olt0 != nullptr && total <= kInitOrderMax) {
-        init_kernel<<<1, 1024, 0, s>>>(olt0, rst0, ctr, n, s0, axis0, row0, rows, *order, 1u);
-        return cudaGetLastError();
+        return launch_chained(init_kernel, 1, 1024, 0, s, olt0, rst0, ctr, n, s0, axis0, row0, rows, *order, 1u);
     }
     uint32_t blocks = (total + 255u) / 256u;
     if (blocks < 1)
         blocks = 1;
     if (blocks > 4096)
         blocks = 4096;
-    init_kernel<<<blocks, 256, 0, s>>>(olt0, rst0, ctr, n, s0, axis0, row0, rows, PixelMap{}, 0u);
-    return cudaGetLastError();
+    return launch_chained(init_kernel, (int)blocks, 256, 0, s, olt0, rst0, ctr, n, s0, axis0, row0, rows,
+                          PixelMap{}, 0u);
 }
 
 template <bool COUNT, bool BATCH, int NS>
-static void level_launch(const LevelArgs &a, int sms, cudaStream_t s)
+static cudaError_t level_launch(const LevelArgs &a, int sms, cudaStream_t s)
 {
-    const size_t smem = a.exact_last ? (size_t)(256 / 32) * kWarpStage * sizeof(uint32_t) : 0u;
+    const size_t stage = (size_t)(256 / 32) * kWarpStage * sizeof(uint32_t);
+    const size_t smem = a.exact_last ? stage : 0u;
+    static const int plain = resident_ctas(level_kernel<COUNT, BATCH, NS>, 256, 0);
+    static const int staged = resident_ctas(level_kernel<COUNT, BATCH, NS>, 256, stage);
     // no more CTAs than the level can have items for
     const unsigned long long most = ((unsigned long long)a.bound * a.chunks + 7u) / 8u;
-    int grid = persistent_grid(level_kernel<COUNT, BATCH, NS>, 256, smem, sms);
+    int grid = (a.exact_last ? staged : plain) * sms;
     if (most < (unsigned long long)grid)
         grid = most ? (int)most : 1;
-    level_kernel<COUNT, BATCH, NS><<<grid, 256, smem, s>>>(a);
+    return launch_chained(level_kernel<COUNT, BATCH, NS>, grid, 256, smem, s, a);
 }
 
 cudaError_t launch_level(const LevelArgs &a, bool count, bool batch, int sms, cudaStream_t s)
@@ -861,25 +858,21 @@ cudaError_t launch_level(const LevelArgs &a, bool count, bool batch, int sms, cu
     const bool two = a.chunks > 1u || a.side > kLevelSide1;
     if (batch) {
         if (count)
-            two ? level_launch<true, true, 2>(a, sms, s) : level_launch<true, true, 1>(a, sms, s);
-        else
-            two ? level_launch<false, true, 2>(a, sms, s) : level_launch<false, true, 1>(a, sms, s);
-    } else {
-        if (count)
-            two ? level_launch<true, false, 2>(a, sms, s) : level_launch<true, false, 1>(a, sms, s);
-        else
-            two ? level_launch<false, false, 2>(a, sms, s) : level_launch<false, false, 1>(a, sms, s);
+            return two ? level_launch<true, true, 2>(a, sms, s) : level_launch<true, true, 1>(a, sms, s);
+        return two ? level_launch<false, true, 2>(a, sms, s) : level_launch<false, true, 1>(a, sms, s);
     }
-    return cudaGetLastError();
+    if (count)
+        return two ? level_launch<true, false, 2>(a, sms, s) : level_launch<true, false, 1>(a, sms, s);
+    return two ? level_launch<false, false, 2>(a, sms, s) : level_launch<false, false, 1>(a, sms, s);
 }
 
 cudaError_t launch_fill(const FillArgs &f, bool batch, int sms, cudaStream_t s)
 {
     if (batch) {
-        const int grid = persistent_grid(fill_kernel<true>, 256, 0, sms);
+        const int grid = resident_ctas(fill_kernel<true>, 256, 0) * sms;
         fill_kernel<true><<<grid, 256, 0, s>>>(f);
     } else {
-        const int grid = persistent_grid(fill_kernel<false>, 256, 0, sms);
+        const int grid = resident_ctas(fill_kernel<false>, 256, 0) * sms;
         fill_kernel<false><<<grid, 256, 0, s>>>(f);
     }
     return cudaGetLastError();
@@ -888,20 +881,20 @@ cudaError_t launch_fill(const FillArgs &f, bool batch, int sms, cudaStream_t s)
 cudaError_t launch_init_batch(uint4 *olt0, uint4 *rst0, DevCounters *ctr, const FrameDesc *frames,
                               uint32_t nframes, uint32_t total0, cudaStream_t s)
 {
-    init_batch_kernel<<<nframes, 256, 0, s>>>(olt0, rst0, ctr, frames, total0);
-    return cudaGetLastError();
+    return launch_chained(init_batch_kernel, (int)nframes, 256, 0, s, olt0, rst0, ctr, frames, total0);
 }
 
 template <bool COUNT, bool BATCH>
-static void refill_launch(const LeafArgs &a, int sms, cudaStream_t s)
+static cudaError_t refill_launch(const LeafArgs &a, int sms, cudaStream_t s)
 {
     const int threads = kRefillWarps * 32;
     // no more CTAs than the leaves can have pre-passes for
     const unsigned long long most = a.bound * a.side * a.side / (64u * kRefillWarps) + 1u;
-    int grid = persistent_grid(leaf_refill_kernel<COUNT, BATCH>, threads, 0, sms);
+    static const int resident = resident_ctas(leaf_refill_kernel<COUNT, BATCH>, threads, 0);
+    int grid = resident * sms;
     if (most < (unsigned long long)grid)
         grid = (int)most;
-    leaf_refill_kernel<COUNT, BATCH><<<grid, threads, 0, s>>>(a);
+    return launch_chained(leaf_refill_kernel<COUNT, BATCH>, grid, threads, 0, s, a);
 }
 
 cudaError_t launch_leaf(const LeafArgs &a, uint32_t bx, uint32_t by, bool count, bool tiled,
@@ -910,27 +903,18 @@ cudaError_t launch_leaf(const LeafArgs &a, uint32_t bx, uint32_t by, bool count,
     if (batch) {
         if (tiled)
             return cudaErrorInvalidValue;
-        if (count)
-            refill_launch<true, true>(a, sms, s);
-        else
-            refill_launch<false, true>(a, sms, s);
-        return cudaGetLastError();
+        return count ? refill_launch<true, true>(a, sms, s) : refill_launch<false, true>(a, sms, s);
     }
-    if (!tiled) {
-        if (count)
-            refill_launch<true, false>(a, sms, s);
-        else
-            refill_launch<false, false>(a, sms, s);
-        return cudaGetLastError();
-    }
+    if (!tiled)
+        return count ? refill_launch<true, false>(a, sms, s) : refill_launch<false, false>(a, sms, s);
     const uint32_t tiles_x = (a.side + bx - 1) / bx, tiles_y = (a.side + by - 1) / by;
     const dim3 block(bx, by);
     const int threads = (int)(bx * by);
     if (count) {
-        const int grid = persistent_grid(leaf_kernel<true>, threads, 0, sms);
+        const int grid = resident_ctas(leaf_kernel<true>, threads, 0) * sms;
         leaf_kernel<true><<<grid, block, 0, s>>>(a, a.leaf_cap, tiles_x, tiles_x * tiles_y);
     } else {
-        const int grid = persistent_grid(leaf_kernel<false>, threads, 0, sms);
+        const int grid = resident_ctas(leaf_kernel<false>, threads, 0) * sms;
         leaf_kernel<false><<<grid, block, 0, s>>>(a, a.leaf_cap, tiles_x, tiles_x * tiles_y);
     }
     return cudaGetLastError();
