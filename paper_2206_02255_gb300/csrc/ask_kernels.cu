@@ -668,7 +668,7 @@ __global__ void __launch_bounds__(1024) leaf_kernel(LeafArgs a, uint32_t leaf_ca
 //    ring of survivors in shared memory.  Most pixels end here, with no
 //    per-pixel bookkeeping beyond the lane they run on;
 //  * refill loop over the survivors: each lane carries two orbits; every
-//    round each orbit runs one unchecked block of kLeafUnroll updates; an
+//    round each orbit runs two unchecked blocks of kLeafUnroll updates; an
 //    orbit that escaped (or has less than a block left) waits at the block's
 //    start until kRefillSlots slots wait or are idle; then the waiting ones
 //    go to the warp's park buffer and the free slots take the next survivors

@@ -175,7 +175,10 @@ constexpr int kSlots = 2;          // orbits per lane in the refill loop (four: 
 constexpr uint32_t kParkCap = 96;  // parked orbits per warp (fewer than 32 wait, a round adds 64)
 constexpr uint32_t kRingCap = 96;  // survivors per warp (< 32 + 64: topped up while below 32)
 constexpr uint32_t kRawCount = 0xffffffffu;  // count of an orbit that may not run in blocks
-constexpr int kLeafUnroll = 64;    // updates per unchecked block of the refill loop (a power of two)
+constexpr int kLeafUnroll = 32;    // updates per unchecked block of the refill loop (a power of
+                                   // two), two blocks a round: with one block of 64 an orbit
+                                   // that escapes is searched for 31 updates instead of 15
+                                   // (64 frames in a batch: 38.8 ms against 38.0)
 // Idle or waiting slots (of 64) before a warp parks and refills: that code
 // costs about a third of a round, and most rounds end a few orbits.  At
 // n = 16384 the leaf kernel took 1.097 ms with 1, 1.077 with 8, 1.095 with 16.
@@ -207,6 +210,13 @@ __device__ __forceinline__ LView leaf_view(const LeafArgs &a, uint32_t frame)
         v.max_dwell = a.max_dwell;
     }
     return v;
+}
+
+template <bool BATCH>
+__device__ __forceinline__ void store_dwell(const LeafArgs &a, uint32_t frame, uint32_t pix, uint32_t v)
+{
+    const LView f = leaf_view<BATCH>(a, frame);
+    f.map[(size_t)(pix >> 16) * f.n + (pix & 0xffffu)] = v;
 }
 
 // Exact dwell of a parked orbit: s.xy = state after d updates, known to
@@ -612,16 +622,14 @@ __device__ __forceinline__ uint32_t pre_pass(const LeafArgs &a, Src &src, uint32
             r1 += m1 < 4.0f ? h : 0u;
         }
         if (esc0) {
-            const LView v = leaf_view<BATCH>(a, fr0);
-            v.map[(size_t)(pix0 >> 16) * v.n + (pix0 & 0xffffu)] = r0 + 1u;
+            store_dwell<BATCH>(a, fr0, pix0, r0 + 1u);
             if (COUNT) {
                 it += r0 + 1u;
                 ++lpx;
             }
         }
         if (esc1) {
-            const LView v = leaf_view<BATCH>(a, fr1);
-            v.map[(size_t)(pix1 >> 16) * v.n + (pix1 & 0xffffu)] = r1 + 1u;
+            store_dwell<BATCH>(a, fr1, pix1, r1 + 1u);
             if (COUNT) {
                 it += r1 + 1u;
                 ++lpx;
@@ -717,10 +725,10 @@ __device__ __forceinline__ void fold_slot1(WarpLeaf<BATCH> &w, WarpFill &f, Slot
     __syncwarp();
 }
 
-// Settle a slot after a block (x, y: the state after it): an orbit
-// that passed the block's test counts it, and is done, at max_dwell, when the
-// block ends there (the block limit lim stands K - 1 below max_dwell) or when
-// its state equals the saved one (bx, by): the iteration is a function of the
+// Settle a slot after a round's second block (x, y: the state after it): an
+// orbit that passed the block's test counts it, and is done, at max_dwell, when
+// it has got there (the block limit lim stands kLeafUnroll - 1 below max_dwell)
+// or when its state equals the saved one (bx, by): the iteration is a function of the
 // state alone, so an orbit that repeats a state repeats it for ever and never
 // escapes.  (Equal up to the sign of a zero, which changes no magnitude and
 // no test.)  The saved state is renewed whenever d / K is a power of two, so a
@@ -732,28 +740,26 @@ template <bool COUNT, bool BATCH>
 __device__ __forceinline__ bool settle_slot(const LeafArgs &a, Slot &s, float x, float y,
                                             unsigned long long &it, unsigned long long &lpx)
 {
-    const uint32_t K = (uint32_t)kLeafUnroll;
+    const uint32_t K = 2u * (uint32_t)kLeafUnroll;
     const uint32_t lim = slot_limit<BATCH>(a, s);
     const bool ok = s.d < lim && z_bounded(x, y);
     if (ok) {
         s.x = x;
         s.y = y;
+        s.d += (uint32_t)kLeafUnroll;
     }
-    if (s.busy && ok) {
-        s.d += K;
-        const uint32_t md = lim + K - 1u;
-        if (s.d == md || (x == s.bx && y == s.by)) {
-            const LView v = leaf_view<BATCH>(a, s.frame);
-            v.map[(size_t)(s.pix >> 16) * v.n + (s.pix & 0xffffu)] = md;
-            if (COUNT) {
-                it += md;
-                ++lpx;
-            }
-            s.busy = false;
-        } else if (((s.d / K) & (s.d / K - 1u)) == 0u) {
-            s.bx = x;
-            s.by = y;
+    const uint32_t md = lim + (uint32_t)kLeafUnroll - 1u;
+    const bool end = s.busy && lim != 0u && s.d == md;
+    if (end || (s.busy && ok && x == s.bx && y == s.by)) {
+        store_dwell<BATCH>(a, s.frame, s.pix, md);
+        if (COUNT) {
+            it += md;
+            ++lpx;
         }
+        s.busy = false;
+    } else if (ok && ((s.d / K) & (s.d / K - 1u)) == 0u) {
+        s.bx = x;
+        s.by = y;
     }
     return s.busy && !ok;
 }
@@ -777,9 +783,10 @@ __device__ __forceinline__ void half_block(float *x, float *y, const float *cr, 
     }
 }
 
-// One round of the refill loop: an unchecked block of kLeafUnroll updates on
-// the first NS slots (the results of an idle slot are not used), and what
-// follows for each slot (settle_slot).  Once `thr` slots or more are idle or
+// One round of the refill loop: two unchecked blocks of kLeafUnroll updates on
+// the first NS slots (the results of an idle slot are not used; an orbit that
+// fails the first block repeats it as its second), and what follows for each
+// slot (settle_slot).  Once `thr` slots or more are idle or
 // wait, the waiting orbits are parked (the state before the block and the
 // block's midpoint state go to the park buffer), and whenever 32 orbits are
 // parked the warp finishes them together.  Returns whether `thr` was reached.
@@ -795,6 +802,20 @@ __device__ __forceinline__ bool refill_round(const LeafArgs &a, WarpLeaf<BATCH> 
         y[i] = s[i].y;
         cr[i] = s[i].cr;
         ci[i] = s[i].ci;
+    }
+    // first block: an orbit that passes it moves on, another repeats it below
+    half_block<NS>(x, y, cr, ci);
+    half_block<NS>(x, y, cr, ci);
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        if (s[i].d < slot_limit<BATCH>(a, s[i]) && z_bounded(x[i], y[i])) {
+            s[i].x = x[i];
+            s[i].y = y[i];
+            s[i].d += (uint32_t)kLeafUnroll;
+        } else {
+            x[i] = s[i].x;
+            y[i] = s[i].y;
+        }
     }
     half_block<NS>(x, y, cr, ci);
 #pragma unroll
