@@ -921,6 +921,7 @@ ask_status enqueue_batch(ask_ctx *ctx, const BatchBuffers &b, const BatchPlan &b
         a.in_cap = (i == 0) ? bp.total0 : (uint32_t)bp.level_cap[i];
         a.out_cap = (i + 1 < bp.L) ? (uint32_t)bp.level_cap[i + 1] : 0u;
         a.bound = bp.level_cap[i];
+        a.side = bp.max_side[i];
         a.chunks = bp.chunks[i];
         a.next_chunks = (i + 1 < bp.L) ? bp.chunks[i + 1] : 1u;
         a.rst_in = b.rst[i & 1];

@@ -359,6 +359,9 @@ enum : uint32_t {
 // early, so the long ones serve orbits that run long (32 at n = 16384: levels 2
 // and 3 at 190 and 387 us against 190 and 371).
 constexpr uint32_t kQueryRound = 64;
+// Whole perimeters of small regions in a batch (zoomed frames, whose orbits all
+// outlive the short rounds): blocks of this size from the first round.
+constexpr uint32_t kQueryRoundBatch = 32;
 // The CTA-wide query of the paper's SBR / MBR mappings: blocks of 32 from
 // the first round.
 constexpr uint32_t kQueryRoundCta = 32;
@@ -648,14 +651,14 @@ __device__ __forceinline__ bool resolve_block(const float *x0, const float *y0, 
 // them about 15 updates where a K-update block and its search cost 2K - 1.
 // The rounds end as soon as an orbit escapes: if another still runs, or never
 // will escape, two dwells differ; else all escaped in this round and their
-// dwells are resolved.  An orbit is proven to stay (its dwell is max_dwell)
+// dwells are resolved.  PROVE: an orbit is proven to stay (its dwell is max_dwell)
 // when it enters its capture disc or repeats the state it had at rounds 1, 2,
 // 4, 8, ... of the long ones, so a cycle is seen within twice the rounds it
 // took to enter it.  w: the region's common dwell as far as known (kNone32:
 // none yet); orbits stop at w + 1.  ps (or NULL): the region's shared state
 // {common dwell, differs}, read along the way, `lag` rounds between a load and
 // its use.  On GROUP_SAME d holds the dwells (above w: anything above w).
-template <uint32_t K, int NS>
+template <uint32_t K, int NS, bool PROVE>
 __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max_dwell,
                                                 const uint32_t *px, const uint32_t *py,
                                                 const bool *active, uint32_t rnd, uint32_t w,
@@ -713,7 +716,7 @@ __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max
                     d[i] = n;
             return GROUP_SAME;
         }
-        if (rnd >= 3u && ((rnd - 3u) & (rnd - 4u)) == 0u) {
+        if (PROVE && rnd >= 3u && ((rnd - 3u) & (rnd - 4u)) == 0u) {
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
                 bx[i] = x[i];
@@ -745,7 +748,7 @@ __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max
                 y[i] = ty[i];
             }
             const float ux = x[i] - ax[i], uy = y[i] - ay[i];
-            const bool in = rnd >= 3u && (__fmaf_rn(ux, ux, __fmul_rn(uy, uy)) < r2[i] ||
+            const bool in = PROVE && rnd >= 3u && (__fmaf_rn(ux, ux, __fmul_rn(uy, uy)) < r2[i] ||
                                           (x[i] == bx[i] && y[i] == by[i]));
             if (run[i] && ok)
                 d[i] = in ? max_dwell : n;
@@ -804,7 +807,7 @@ __device__ __forceinline__ void group_range(const bool *active, const uint32_t *
 
 // Group j of the `groups` of 32 * NS pixels that cover the perimeter of g (P
 // pixels), spread over all of it: pixels j, j + groups, j + 2 groups, ...
-template <uint32_t K, int NS>
+template <uint32_t K, int NS, bool PROVE>
 __device__ __forceinline__ uint32_t spread_group(const PixelMap &pm, uint32_t max_dwell, const Region &g,
                                                  uint32_t first, uint32_t stride, uint32_t base,
                                                  uint32_t P, uint32_t rnd, uint32_t w,
@@ -822,7 +825,7 @@ __device__ __forceinline__ uint32_t spread_group(const PixelMap &pm, uint32_t ma
         if (active[i])
             perimeter_pixel(g, k, px[i], py[i]);
     }
-    const uint32_t r = query_group<K, NS>(pm, max_dwell, px, py, active, rnd, w, ps, lag, lane, d);
+    const uint32_t r = query_group<K, NS, PROVE>(pm, max_dwell, px, py, active, rnd, w, ps, lag, lane, d);
 #pragma unroll
     for (int i = 0; i < NS; ++i)
         if (active[i])
@@ -835,16 +838,16 @@ __device__ __forceinline__ uint32_t spread_group(const PixelMap &pm, uint32_t ma
 // One warp queries the whole perimeter of g, NS orbits a lane.  Returns true
 // and the common dwell in *w_out if the perimeter is uniform; `it` gains the
 // updates made.
-template <uint32_t K, int NS>
+template <uint32_t K, int NS, bool PROVE>
 __device__ __forceinline__ bool warp_perimeter_uniform(const PixelMap &pm, uint32_t max_dwell,
-                                                       const Region &g, uint32_t lane,
+                                                       const Region &g, uint32_t lane, uint32_t rnd,
                                                        uint32_t *w_out, unsigned long long &it)
 {
     const uint32_t P = perimeter_size(g.w, g.h);
     const uint32_t groups = (P + 32u * NS - 1u) / (32u * NS);
     uint32_t w = kNone32, vmin = 0, vmax = 0;
     for (uint32_t j = 0; j < groups; ++j) {
-        const uint32_t r = spread_group<K, NS>(pm, max_dwell, g, j, groups, 0u, P, 0u, w, nullptr, 0u, lane,
+        const uint32_t r = spread_group<K, NS, PROVE>(pm, max_dwell, g, j, groups, 0u, P, rnd, w, nullptr, 0u, lane,
                                                vmin, vmax, it);
         if (r != GROUP_SAME || vmin != vmax || (w != kNone32 && vmin != w))
             return false;

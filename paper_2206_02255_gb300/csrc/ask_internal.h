@@ -107,7 +107,7 @@ struct LevelArgs {
     uint32_t n;
     PixelMap pm;
     uint32_t max_dwell;
-    uint32_t side;        // nominal side of this level's regions
+    uint32_t side;        // nominal side of this level's regions (a batch: the largest)
     uint32_t split;       // non-uniform regions split (else become leaves)
     uint32_t child_side;  // ceil(side / r)
     uint32_t r;

@@ -337,6 +337,28 @@ __device__ __forceinline__ void chunk_exact(const FView &a, const Region &g, uin
     }
 }
 
+// A warp's counts of a level (COUNT mode).
+__device__ __forceinline__ void count_level(const LevelArgs &a, unsigned long long it, unsigned long long bpx,
+                                            unsigned long long fpx, unsigned long long dpx, uint32_t lane)
+{
+    it = warp_sum_u64(it);
+    bpx = warp_sum_u64(bpx);
+    fpx = warp_sum_u64(fpx);
+    dpx = warp_sum_u64(dpx);
+    if (lane == 0) {
+        if (it) {
+            atomicAdd(&a.ctr->iterations, it);
+            atomicAdd(&a.ctr->level_iters[a.level], it);
+        }
+        if (bpx)
+            atomicAdd(&a.ctr->border_pixels, bpx);
+        if (fpx)
+            atomicAdd(&a.ctr->fill_pixels, fpx);
+        if (dpx)
+            atomicAdd(&a.ctr->deferred_fill_pixels, dpx);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Level kernel: one warp per work item (a region, or a perimeter chunk of a
 // large region), NS perimeter orbits a lane.
@@ -360,6 +382,16 @@ constexpr int kLevelMinBlocks1 = 4;
 constexpr int kLevelMinBlocks2 = 3;
 // Level kernels of regions up to this side take one orbit a lane.
 constexpr uint32_t kLevelSide1 = 17;
+// Levels that hold at most this many regions, of perimeters one CTA can take
+// at a time, run one CTA per region (level_cta_kernel).  None / 512 / 2048 /
+// 8192: n = 1024 71 / 66 / 60 / 60 us, n = 2048 179 / 165 / 159 / 155, n = 1999
+// without chunks 278 / 195 / 195 / 201, n = 3001 385 / 386 / 370 / 370.
+constexpr unsigned long long kCtaLevelRegions = 2048;
+// Small regions (one orbit a lane) look for orbits that stay only where a
+// region is at least this wide in the plane: nearer to the boundary proofs come
+// too late to pay for the looks (sides of 16 at n = 16384: 374 us with, 366
+// without; at n = 4096: 82 with, 96 without).
+constexpr float kProveExtent = 0.004f;
 // A ticket of cheap regions stands for at most kTicketMax of them, as long as
 // every warp gets kTicketsPerWarp tickets (1 at most: 377 us at level 3 of n =
 // 16384 and 11.0 ms at n = 65536 against 371 and 10.0; a ticket of several
@@ -367,7 +399,7 @@ constexpr uint32_t kLevelSide1 = 17;
 constexpr uint32_t kTicketMax = 8;
 constexpr uint32_t kTicketsPerWarp = 4;
 
-template <bool COUNT, bool BATCH, int NS>
+template <bool COUNT, bool BATCH, int NS, bool PROVE>
 __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlocks2)
     level_kernel(LevelArgs a)
 {
@@ -466,8 +498,8 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
             if (COUNT && lane == 0)
                 bpx += P;
             if (query) {
-                uniform = warp_perimeter_uniform<kQueryRound, NS>(
-                    f.pm, f.max_dwell, g, lane, &wv, it);
+                uniform = warp_perimeter_uniform<BATCH ? kQueryRoundBatch : kQueryRound, NS, PROVE>(
+                    f.pm, f.max_dwell, g, lane, BATCH ? 3u : 0u, &wv, it);
             } else {
                 // last level, exact perimeters staged in shared memory: a leaf
                 // keeps them and the leaf kernel skips them
@@ -504,7 +536,7 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
             if (COUNT && lane == 0 && c == 0)
                 bpx += P;
             if (query) {
-                const uint32_t r = chunk_query<BATCH, NS>(f, g, P, c, chunks, st, lane, it);
+                const uint32_t r = chunk_query<NS>(f, g, P, c, chunks, st, BATCH ? 1u : kPollLag, lane, it);
                 decided = chunk_decides(r, st, chunks, lane, uniform, wv);
             } else {
                 const uint32_t CP = ceil_div_u32(P, chunks);
@@ -563,24 +595,72 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
     }
     if (j)
         flush_batch<BATCH>(a, b, lane);
-    if (COUNT) {
-        it = warp_sum_u64(it);
-        bpx = warp_sum_u64(bpx);
-        fpx = warp_sum_u64(fpx);
-        dpx = warp_sum_u64(dpx);
-        if (lane == 0) {
-            if (it) {
-                atomicAdd(&a.ctr->iterations, it);
-                atomicAdd(&a.ctr->level_iters[a.level], it);
-            }
-            if (bpx)
-                atomicAdd(&a.ctr->border_pixels, bpx);
-            if (fpx)
-                atomicAdd(&a.ctr->fill_pixels, fpx);
-            if (dpx)
-                atomicAdd(&a.ctr->deferred_fill_pixels, dpx);
+    if (COUNT)
+        count_level(a, it, bpx, fpx, dpx, lane);
+}
+
+// ---------------------------------------------------------------------------
+// Level kernel of a level of few regions: one CTA per region, its warps each a
+// chunk of the perimeter (spread over all of it, two orbits a lane).  The
+// region's query state lives in shared memory and the decision follows a
+// barrier, so a region costs no ticket, no fences and no state in global
+// memory, and the whole CTA fills it.
+// ---------------------------------------------------------------------------
+template <bool COUNT, bool BATCH>
+__global__ void __launch_bounds__(256, kLevelMinBlocks2) level_cta_kernel(LevelArgs a)
+{
+    using R = Rec<BATCH>;
+    using T = typename R::T;
+    __shared__ uint4 st;
+    chain_start();
+    const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+    const uint32_t front = min(a.ctr->count[a.level], a.in_cap);
+    const uint32_t count = front + min(a.ctr->back[a.level], a.in_cap - front);
+    if (blockIdx.x == 0 && threadIdx.x == 0 &&
+        (unsigned long long)a.ctr->count[a.level] + a.ctr->back[a.level] > a.in_cap)
+        atomicOr(&a.ctr->error, ERR_OLT_OVERFLOW);
+    unsigned long long it = 0, bpx = 0, fpx = 0, dpx = 0;
+    for (uint32_t li = blockIdx.x; li < count; li += gridDim.x) {
+        const T e = static_cast<const T *>(a.olt_in)[table_slot(li, front, a.in_cap)];
+        const Region g = R::region(e);
+        const FView f = BATCH ? view_frame(a.frames, R::frame(e), a.level) : view_single(a);
+        const uint32_t P = perimeter_size(g.w, g.h);
+        if (threadIdx.x == 0) {
+            st = make_uint4(kNone, 0u, 0u, 0u);
+            if (COUNT)
+                bpx += P;
         }
+        __syncthreads();
+        chunk_query<2>(f, g, P, wib, blockDim.x / 32u, &st, 1u, lane, it);
+        __syncthreads();
+        const bool uniform = st.y == 0u;
+        const uint32_t wv = st.x;
+        uint32_t kind = f.split ? KIND_SPLIT : KIND_LEAF;
+        if (uniform) {
+            const uint32_t area = g.w * g.h;
+            kind = (a.fills != nullptr && area > kInPlaceFillArea) ? KIND_FILL_LATER : KIND_FILL;
+            if (kind == KIND_FILL)
+                fill_rect(f.map, f.n, g, wv, threadIdx.x, blockDim.x);
+            if (COUNT && threadIdx.x == 0) {
+                fpx += area;
+                if (kind == KIND_FILL_LATER)
+                    dpx += area;
+            }
+        }
+        if (wib == 0) {
+            WarpBatch<BATCH> b;
+            b.rec = e;
+            b.kind = lane == 0 ? kind : KIND_NONE;
+            b.dwell = wv;
+            b.sc = f.child_side;
+            b.r = f.r;
+            b.nchild = (lane == 0 && kind == KIND_SPLIT) ? child_count(g, f.child_side, f.r) : 0u;
+            flush_batch<BATCH>(a, b, lane);
+        }
+        __syncthreads();  // st is free for the next region
     }
+    if (COUNT)
+        count_level(a, it, bpx, fpx, dpx, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -838,32 +918,42 @@ cudaError_t launch_init(uint2 *olt0, uint4 *rst0, DevCounters *ctr, uint32_t n, 
                           PixelMap{}, 0u);
 }
 
-template <bool COUNT, bool BATCH, int NS>
+template <bool COUNT, bool BATCH, int NS, bool PROVE>
 static cudaError_t level_launch(const LevelArgs &a, int sms, cudaStream_t s)
 {
     const size_t stage = (size_t)(256 / 32) * kWarpStage * sizeof(uint32_t);
     const size_t smem = a.exact_last ? stage : 0u;
-    static const int plain = resident_ctas(level_kernel<COUNT, BATCH, NS>, 256, 0);
-    static const int staged = resident_ctas(level_kernel<COUNT, BATCH, NS>, 256, stage);
-    // no more CTAs than the level can have items for
-    const unsigned long long most = ((unsigned long long)a.bound * a.chunks + 7u) / 8u;
+    static const int plain = resident_ctas(level_kernel<COUNT, BATCH, NS, PROVE>, 256, 0);
+    static const int staged = resident_ctas(level_kernel<COUNT, BATCH, NS, PROVE>, 256, stage);
+    // no more CTAs than the level can have items for, but one an SM as long as
+    // there is an item for each
+    const unsigned long long items = a.bound * a.chunks;
+    const unsigned long long most = std::max((items + 7u) / 8u, std::min(items, (unsigned long long)sms));
     int grid = (a.exact_last ? staged : plain) * sms;
     if (most < (unsigned long long)grid)
         grid = most ? (int)most : 1;
-    return launch_chained(level_kernel<COUNT, BATCH, NS>, grid, 256, smem, s, a);
+    return launch_chained(level_kernel<COUNT, BATCH, NS, PROVE>, grid, 256, smem, s, a);
+}
+
+template <bool COUNT, bool BATCH>
+static cudaError_t level_launch_sized(const LevelArgs &a, int sms, cudaStream_t s)
+{
+    const bool query_all = !a.exact_last || (!BATCH && a.split != 0u);
+    if (a.bound <= kCtaLevelRegions && query_all && (a.chunks <= 8u || a.rst_in == nullptr))
+        return launch_chained(level_cta_kernel<COUNT, BATCH>, std::max(1, (int)a.bound),
+                              32 * (int)std::min(8u, std::max(1u, (4u * a.side + 63u) / 64u)), 0, s, a);
+    if (a.chunks > 1u || (!BATCH && a.side > kLevelSide1))
+        return level_launch<COUNT, BATCH, 2, true>(a, sms, s);
+    if (!BATCH && (float)a.side * std::max(a.pm.dx, a.pm.dy) >= kProveExtent)
+        return level_launch<COUNT, BATCH, 1, true>(a, sms, s);
+    return level_launch<COUNT, BATCH, 1, false>(a, sms, s);
 }
 
 cudaError_t launch_level(const LevelArgs &a, bool count, bool batch, int sms, cudaStream_t s)
 {
-    const bool two = a.chunks > 1u || a.side > kLevelSide1;
-    if (batch) {
-        if (count)
-            return two ? level_launch<true, true, 2>(a, sms, s) : level_launch<true, true, 1>(a, sms, s);
-        return two ? level_launch<false, true, 2>(a, sms, s) : level_launch<false, true, 1>(a, sms, s);
-    }
-    if (count)
-        return two ? level_launch<true, false, 2>(a, sms, s) : level_launch<true, false, 1>(a, sms, s);
-    return two ? level_launch<false, false, 2>(a, sms, s) : level_launch<false, false, 1>(a, sms, s);
+    if (batch)
+        return count ? level_launch_sized<true, true>(a, sms, s) : level_launch_sized<false, true>(a, sms, s);
+    return count ? level_launch_sized<true, false>(a, sms, s) : level_launch_sized<false, false>(a, sms, s);
 }
 
 cudaError_t launch_fill(const FillArgs &f, bool batch, int sms, cudaStream_t s)

@@ -236,10 +236,10 @@ __device__ __forceinline__ void process_item(const QueueArgs &q, uint32_t t, uin
     uint32_t wv = 0;
     if (C <= 1u) {
         decided = true;
-        uniform = warp_perimeter_uniform<kQueryRound, 1>(f.pm, f.max_dwell, g, lane, &wv, it);
+        uniform = warp_perimeter_uniform<kQueryRoundBatch, 1, false>(f.pm, f.max_dwell, g, lane, 3u, &wv, it);
     } else {
         uint4 *st = q.rst + aux;
-        decided = chunk_decides(chunk_query<true, 1>(f, g, P, c, C, st, lane, it), st, C, lane, uniform, wv);
+        decided = chunk_decides(chunk_query<1>(f, g, P, c, C, st, 1u, lane, it), st, C, lane, uniform, wv);
     }
     if (COUNT) {
         it = warp_sum_u64(it);

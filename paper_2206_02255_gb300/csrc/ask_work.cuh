@@ -98,15 +98,15 @@ constexpr uint32_t kShortRoundsMaxPerimeter = 512;
 // one of them has set y.  Returns whether this chunk found the difference
 // first (GROUP_DIFFER: the caller decides the region), found none
 // (GROUP_SAME), or stopped because another did (GROUP_STOP).
-template <bool BATCH, int NS>
+template <int NS>
 __device__ __forceinline__ uint32_t chunk_query(const FView &a, const Region &g, uint32_t P, uint32_t c,
-                                                uint32_t chunks, uint4 *st, uint32_t lane,
-                                                unsigned long long &it)
+                                                uint32_t chunks, uint4 *st, uint32_t lag,
+                                                uint32_t lane, unsigned long long &it)
 {
     const volatile uint32_t *ps = reinterpret_cast<const volatile uint32_t *>(st);
     const uint32_t n = P > c ? (P - c + chunks - 1u) / chunks : 0u;
     const uint32_t rnd = P <= kShortRoundsMaxPerimeter ? 0u : 3u;
-    constexpr uint32_t K = kQueryRound, lag = BATCH ? 1u : kPollLag;
+    constexpr uint32_t K = kQueryRound;
     for (uint32_t base = 0; base < n; base += 32u * NS) {
         uint32_t sx = 0, sy = 0, vmin = 0, vmax = 0;
         if (lane == 0) {
@@ -116,7 +116,7 @@ __device__ __forceinline__ uint32_t chunk_query(const FView &a, const Region &g,
         if (__shfl_sync(kFull, sy, 0))
             return GROUP_STOP;
         sx = __shfl_sync(kFull, sx, 0);
-        const uint32_t r = spread_group<K, NS>(a.pm, a.max_dwell, g, c, chunks, base, P, rnd, sx, ps, lag,
+        const uint32_t r = spread_group<K, NS, true>(a.pm, a.max_dwell, g, c, chunks, base, P, rnd, sx, ps, lag,
                                                lane, vmin, vmax, it);
         if (r == GROUP_STOP)
             return r;
