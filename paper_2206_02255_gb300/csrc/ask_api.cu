@@ -24,6 +24,10 @@ struct BatchBuffers {
     uint64_t rst_cap = 0;
     uint4 *fills = nullptr;
     uint64_t fill_cap = 0;
+    float4 *pool = nullptr;              // survivors of a small batch
+    uint64_t pool_cap = 0;
+    uint32_t *pool_f = nullptr;
+    uint64_t pool_f_cap = 0;
     ask::FrameDesc *frames = nullptr;    // device frame table
     uint64_t frames_cap = 0;
     ask::DevCounters *ctr = nullptr;     // not owned when it is the context's
@@ -682,6 +686,9 @@ ask_status render_impl(ask_ctx *ctx, ask_method method, const ask_window *window
     la.skip_perimeter = exact ? 1u : 0u;
     la.fills = fused ? ctx->fills : nullptr;
     la.fill_cap = fused ? (uint32_t)ctx->fill_cap : 0u;
+    la.pool = nullptr;
+    la.pool_frame = nullptr;
+    la.pool_cap = 0u;
     la.ctr = ctx->ctr;
     if (sbr)
         e = launch_leaf_region(la, p.block_x, p.block_y, count, sms, s);
@@ -736,6 +743,7 @@ struct BatchPlan {
     uint64_t level_cap[ASK_MAX_LEVELS] = {};  // bound on each level's regions over the frames
     uint32_t total0 = 0;
     uint32_t leaf_side = 0;               // largest nominal leaf side over the frames
+    uint64_t pixels = 0;                  // of all frames
     // the persistent batch kernel: queue items (every level's chunk items and
     // fill bands of every frame), chunk states, level-0 items and states
     uint64_t q_items = 0, q_states = 0, q_total0 = 0, q_states0 = 0;
@@ -812,6 +820,7 @@ ask_status plan_batch(ask_ctx *ctx, const ask_frame *frames, uint32_t nframes, u
         if (d.chunks[0] > 1u)
             bp.q_states0 += regions0;
         bp.leaf_need += plan.max_regions[plan.levels - 1];
+        bp.pixels += (uint64_t)fr.n * fr.n;
         bp.leaf_side = std::max(bp.leaf_side, plan.side[plan.levels - 1]);
         total0 += (uint64_t)plan.axis0 * plan.axis0;
         if (plan.levels > bp.L)
@@ -866,6 +875,10 @@ ask_status reserve_batch(ask_ctx *ctx, BatchBuffers &b, const BatchPlan &bp, boo
         return st;
     if ((st = grow(ctx, &b.fills, &b.fill_cap, bp.fill_need, "cudaMalloc(batch fills)")) != ASK_OK)
         return st;
+    const uint64_t pool = pool_need(bp.pixels);
+    if ((st = grow(ctx, &b.pool, &b.pool_cap, pool, "cudaMalloc(survivor pool)")) != ASK_OK ||
+        (st = grow(ctx, &b.pool_f, &b.pool_f_cap, pool, "cudaMalloc(survivor pool)")) != ASK_OK)
+        return st;
     if ((st = grow(ctx, &b.frames, &b.frames_cap, (uint64_t)bp.desc.size(), "cudaMalloc(frame table)")) !=
         ASK_OK)
         return st;
@@ -891,6 +904,10 @@ void free_batch(BatchBuffers &b, bool own_counters)
         cudaFree(b.leaves);
     if (b.fills)
         cudaFree(b.fills);
+    if (b.pool)
+        cudaFree(b.pool);
+    if (b.pool_f)
+        cudaFree(b.pool_f);
     if (b.frames)
         cudaFree(b.frames);
     if (own_counters && b.ctr)
@@ -947,11 +964,15 @@ ask_status enqueue_batch(ask_ctx *ctx, const BatchBuffers &b, const BatchPlan &b
     la.bound = bp.leaf_need;
     la.side = bp.leaf_side;
     la.skip_perimeter = exact ? 1u : 0u;
+    const uint64_t pool = pool_need(bp.pixels);
+    la.pool = pool ? b.pool : nullptr;
+    la.pool_frame = pool ? b.pool_f : nullptr;
+    la.pool_cap = (uint32_t)pool;
     la.frames = b.frames;
     la.ctr = b.ctr;
     if ((e = launch_leaf(la, 16, 16, count, false, true, sms, s)) != cudaSuccess)
         return cuda_err(ctx, e, "batch leaf kernel");
-    ++n_launch;
+    n_launch += pool ? 2u : 1u;
     if (launches)
         *launches = n_launch;
     return ASK_OK;

@@ -34,6 +34,8 @@ struct DevCounters {
     uint32_t leaf_work;                     // next leaf the leaf kernel hands out
     uint32_t fill_count;                    // bands in the deferred-fill list
     uint32_t fill_work;                     // next band the leaf kernel's fill warps take
+    uint32_t pool_count;                    // survivors put in the pool (may exceed its capacity)
+    uint32_t pool_work;                     // next pool entries handed out
     uint32_t leaf_light;                    // leaf-list entries from the back (level kernels:
                                             // leaves whose probe escaped, taken last)
     uint32_t back[ASK_MAX_LEVELS + 1];      // region-table entries of level i written from the
@@ -191,9 +193,23 @@ struct LeafArgs {
     uint32_t skip_perimeter;  // leaf perimeters are already in the map
     const uint4 *fills;   // lane-refill kernel: deferred-fill bands to write
     uint32_t fill_cap;    //   along the way (NULL: none)
+    // small batches: the survivors of the leaf kernel's pre-passes go to this
+    // pool (state, pixel, count; frame), which a second kernel works through
+    // (NULL: every warp keeps its own)
+    float4 *pool;
+    uint32_t *pool_frame;
+    uint32_t pool_cap;
     const FrameDesc *frames;
     DevCounters *ctr;
 };
+// Batches of at most kPoolPixels pixels in all pool their survivors, up
+// to kPoolEntries of them (those beyond stay with their warps).
+constexpr uint64_t kPoolPixels = 1ull << 24;
+constexpr uint64_t kPoolEntries = 1ull << 22;
+inline uint64_t pool_need(uint64_t pixels)
+{
+    return pixels > kPoolPixels ? 0u : pixels < kPoolEntries ? pixels : kPoolEntries;
+}
 // tiled = false: lane-refill kernel (default); true: one thread per pixel in
 // block_x x block_y tiles (single frame only)
 cudaError_t launch_leaf(const LeafArgs &a, uint32_t bx, uint32_t by, bool count, bool tiled,

@@ -805,55 +805,57 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocks) leaf_refi
     src.extent = &extent;
     uint32_t srcst = SRC_MORE;
     cursor_reset(w.cursor, lane);
-    Slot s[kSlots];
-#pragma unroll
-    for (int i = 0; i < kSlots; ++i)
-        slot_reset(s[i]);
     unsigned long long it = 0, lpx = 0;
-
-    for (;;) {
-        // refill idle slots from the ring, topping it up with pre-passes
-        // while it holds fewer survivors than idle slots (at most 32)
-        for (;;) {
-            const uint32_t idle = 32u * kSlots - busy_slots<kSlots>(s);
-            if (idle < kRefillSlots || (srcst != SRC_MORE && f.ring_n == 0))
-                break;
-            const uint32_t want = min(idle, 32u);
-            while (f.ring_n < want && srcst == SRC_MORE)
-                pre_pass<COUNT, BATCH>(a, src, srcst, w, f, lane, it, lpx);
-            refill_from_ring<BATCH, kSlots>(a, w, f, s);
-        }
-        // once the leaves have run out and the orbits left fit in one slot
-        // per lane, the tail runs on slot 0 alone
-        if (srcst != SRC_MORE && f.ring_n + busy_slots<kSlots>(s) <= 32u)
-            break;
-        while (!refill_round<COUNT, BATCH, kSlots>(a, w, f, s, kRefillSlots, lane, it, lpx)) {
-        }
-    }
-    fold_slot1<BATCH>(w, f, s[1]);
-    refill_from_ring<BATCH, 1>(a, w, f, s);
-    while (!refill_round<COUNT, BATCH, 1>(a, w, f, s, 32u, lane, it, lpx)) {
-    }
+    PrePassFeed<COUNT, BATCH, LeafList<BATCH>> feed{src};
+    // a small batch: pre-passes only, the survivors to the pool while it has room
+    if (BATCH && a.pool != nullptr)
+        do
+            feed(a, srcst, w, f, lane, it, lpx);
+        while (pool_survivors<BATCH>(a, w, f, lane) && srcst == SRC_MORE);
+    if (f.ring_n != 0u || srcst == SRC_MORE)
+        run_orbits<COUNT, BATCH>(a, feed, srcst, w, f, lane, it, lpx);
     if (a.fills != nullptr)
         drain_fills<BATCH>(a, lane);
-    // the orbits still parked
-    if (lane < f.parked) {
-        finish_parked<COUNT, BATCH>(a, w.park_s[lane], w.park_u[lane], BATCH ? w.park_f[lane] : 0u, it);
-        if (COUNT)
-            ++lpx;
-    }
-    if (COUNT) {
-        it = warp_sum_u64(it);
-        lpx = warp_sum_u64(lpx);
-        if (lane == 0) {
-            if (it) {
-                atomicAdd(&a.ctr->iterations, it);
-                atomicAdd(&a.ctr->leaf_iters, it);
-            }
-            if (lpx)
-                atomicAdd(&a.ctr->leaf_pixels, lpx);
-        }
-    }
+    finish_orbits<COUNT, BATCH>(a, w, f, lane, it, lpx);
+}
+
+// ---------------------------------------------------------------------------
+// Second kernel of a small batch's leaves: the pooled survivors, dealt evenly.
+//
+// In the leaf kernel of a small batch a warp that took a few heavy leaves runs
+// on long after the others; pooled, its orbits are dealt to all warps, 32 at a
+// time, and to no more warps than they fill (kPoolPerWarp each, spread over the
+// schedulers), since a round costs the same for 5 lanes as for 64.  12 frames
+// of up to 1024 pixels as a graph: 456 -> 364 us (leaf kernel 265 us; 77 + 117
+// with the pool).  Single frames keep their survivors: their leaves are alike
+// enough, and the second kernel cost more than it gave (n = 3001 362 -> 379 us,
+// n = 1024 60 -> 64 us, n = 4096 354 -> 344 us).
+// ---------------------------------------------------------------------------
+constexpr uint32_t kPoolPerWarp = 64;
+template <bool COUNT>
+__global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocks) pool_kernel(LeafArgs a, uint32_t resident)
+{
+    __shared__ WarpLeaf<true> shared[kRefillWarps];
+    chain_start();
+    const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+    const uint32_t total = min(a.ctr->pool_count, a.pool_cap);
+    // active warps per CTA, rotated from CTA to CTA of an SM so that they
+    // spread over its schedulers
+    const uint32_t per_cta = min((uint32_t)kRefillWarps,
+                                 (total + kPoolPerWarp * gridDim.x - 1u) / (kPoolPerWarp * gridDim.x));
+    const uint32_t rank = (wib + blockIdx.x * resident / gridDim.x) % (uint32_t)kRefillWarps;
+    if (rank >= per_cta)
+        return;
+    WarpLeaf<true> &w = shared[wib];
+    WarpFill f;
+    f.parked = f.ring_h = f.ring_n = 0;
+    PoolFeed feed;
+    feed.total = total;
+    feed.next = kPoolTake * (blockIdx.x + gridDim.x * rank);
+    feed.first_end = kPoolTake * gridDim.x * per_cta;
+    unsigned long long it = 0, lpx = 0;
+    run_orbits<COUNT, true>(a, feed, SRC_MORE, w, f, lane, it, lpx);
+    finish_orbits<COUNT, true>(a, w, f, lane, it, lpx);
 }
 
 // Level-0 records and counters of a batch: block f writes frame f's
@@ -981,10 +983,13 @@ static cudaError_t refill_launch(const LeafArgs &a, int sms, cudaStream_t s)
     // no more CTAs than the leaves can have pre-passes for
     const unsigned long long most = a.bound * a.side * a.side / (64u * kRefillWarps) + 1u;
     static const int resident = resident_ctas(leaf_refill_kernel<COUNT, BATCH>, threads, 0);
-    int grid = resident * sms;
-    if (most < (unsigned long long)grid)
-        grid = (int)most;
-    return launch_chained(leaf_refill_kernel<COUNT, BATCH>, grid, threads, 0, s, a);
+    const int grid = (int)std::min<unsigned long long>(most, (unsigned long long)(resident * sms));
+    const cudaError_t e = launch_chained(leaf_refill_kernel<COUNT, BATCH>, grid, threads, 0, s, a);
+    if (!BATCH || e != cudaSuccess || a.pool == nullptr)
+        return e;
+    static const int pooled = resident_ctas(pool_kernel<COUNT>, threads, 0);
+    const int pgrid = (int)std::min<unsigned long long>(most, (unsigned long long)(pooled * sms));
+    return launch_chained(pool_kernel<COUNT>, pgrid, threads, 0, s, a, (uint32_t)pooled);
 }
 
 cudaError_t launch_leaf(const LeafArgs &a, uint32_t bx, uint32_t by, bool count, bool tiled,

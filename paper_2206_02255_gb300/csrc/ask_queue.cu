@@ -547,6 +547,9 @@ cudaError_t launch_queue(const QueueArgs &q, uint32_t nframes, bool count, int s
     a.skip_perimeter = 0;
     a.fills = nullptr;
     a.fill_cap = 0;
+    a.pool = nullptr;
+    a.pool_frame = nullptr;
+    a.pool_cap = 0;
     a.frames = q.frames;
     a.ctr = q.ctr;
     const int threads = kRefillWarps * 32;

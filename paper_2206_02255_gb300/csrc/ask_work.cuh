@@ -862,4 +862,135 @@ __device__ __forceinline__ bool refill_round(const LeafArgs &a, WarpLeaf<BATCH> 
     return true;
 }
 
+// Move the ring's survivors to the pool; false once the pool is full (what did
+// not fit stays on the ring).
+template <bool BATCH>
+__device__ __forceinline__ bool pool_survivors(const LeafArgs &a, const WarpLeaf<BATCH> &w, WarpFill &f,
+                                               uint32_t lane)
+{
+    uint32_t base = 0;
+    if (lane == 0 && f.ring_n)
+        base = atomicAdd(&a.ctr->pool_count, f.ring_n);
+    base = __shfl_sync(kFull, base, 0);
+    const uint32_t fit = base < a.pool_cap ? min(f.ring_n, a.pool_cap - base) : 0u;
+    for (uint32_t k = lane; k < fit; k += 32u) {
+        uint32_t j = f.ring_h + k;
+        if (j >= kRingCap)
+            j -= kRingCap;
+        a.pool[base + k] = w.ring[j];
+        if (BATCH)
+            a.pool_frame[base + k] = w.ring_f[j];
+    }
+    f.ring_h += fit;
+    if (f.ring_h >= kRingCap)
+        f.ring_h -= kRingCap;
+    f.ring_n -= fit;
+    __syncwarp();
+    return f.ring_n == 0u;
+}
+
+// Survivors from the pool, kPoolTake at a time onto the ring: a warp's first
+// ones by its number, the others by a counter.
+constexpr uint32_t kPoolTake = 32;
+struct PoolFeed {
+    uint32_t total, next, first_end;  // entries; the warp's next; where the counter's begin
+
+    __device__ __forceinline__ void operator()(const LeafArgs &a, uint32_t &srcst, WarpLeaf<true> &w,
+                                               WarpFill &f, uint32_t lane, unsigned long long &,
+                                               unsigned long long &)
+    {
+        if (next == kNone) {
+            if (lane == 0)
+                next = first_end + atomicAdd(&a.ctr->pool_work, kPoolTake);
+            next = __shfl_sync(kFull, next, 0);
+        }
+        if (next >= total) {
+            srcst = SRC_DONE;
+            return;
+        }
+        const uint32_t n = min(kPoolTake, total - next);
+        if (lane < n) {
+            const float4 e = a.pool[next + lane];
+            push_survivor<true>(w, f, lane, e.x, e.y, __float_as_uint(e.z), __float_as_uint(e.w),
+                                a.pool_frame[next + lane]);
+        }
+        f.ring_n += n;
+        next = kNone;
+        __syncwarp();
+    }
+};
+
+// Survivors of pre-passes over the pixels of a source.
+template <bool COUNT, bool BATCH, typename Src>
+struct PrePassFeed {
+    Src &src;
+
+    __device__ __forceinline__ void operator()(const LeafArgs &a, uint32_t &srcst, WarpLeaf<BATCH> &w,
+                                               WarpFill &f, uint32_t lane, unsigned long long &it,
+                                               unsigned long long &lpx)
+    {
+        pre_pass<COUNT, BATCH>(a, src, srcst, w, f, lane, it, lpx);
+    }
+};
+
+// Refill rounds over the survivors that `feed` puts on the ring, until it has
+// run out (srcst) and no orbit is left but the fewer than 32 still parked.
+template <bool COUNT, bool BATCH, typename Feed>
+__device__ __forceinline__ void run_orbits(const LeafArgs &a, Feed &feed, uint32_t srcst,
+                                           WarpLeaf<BATCH> &w, WarpFill &f, uint32_t lane,
+                                           unsigned long long &it, unsigned long long &lpx)
+{
+    Slot s[kSlots];
+#pragma unroll
+    for (int i = 0; i < kSlots; ++i)
+        slot_reset(s[i]);
+    for (;;) {
+        // refill idle slots from the ring, topping it up while it holds fewer
+        // survivors than idle slots (at most 32)
+        for (;;) {
+            const uint32_t idle = 32u * kSlots - busy_slots<kSlots>(s);
+            if (idle < kRefillSlots || (srcst != SRC_MORE && f.ring_n == 0))
+                break;
+            const uint32_t want = min(idle, 32u);
+            while (f.ring_n < want && srcst == SRC_MORE)
+                feed(a, srcst, w, f, lane, it, lpx);
+            refill_from_ring<BATCH, kSlots>(a, w, f, s);
+        }
+        // once the source has run out and the orbits left fit in one slot
+        // per lane, the tail runs on slot 0 alone
+        if (srcst != SRC_MORE && f.ring_n + busy_slots<kSlots>(s) <= 32u)
+            break;
+        while (!refill_round<COUNT, BATCH, kSlots>(a, w, f, s, kRefillSlots, lane, it, lpx)) {
+        }
+    }
+    fold_slot1<BATCH>(w, f, s[1]);
+    refill_from_ring<BATCH, 1>(a, w, f, s);
+    while (!refill_round<COUNT, BATCH, 1>(a, w, f, s, 32u, lane, it, lpx)) {
+    }
+}
+
+// The orbits still parked after run_orbits, and the warp's counts.
+template <bool COUNT, bool BATCH>
+__device__ __forceinline__ void finish_orbits(const LeafArgs &a, const WarpLeaf<BATCH> &w, const WarpFill &f,
+                                              uint32_t lane, unsigned long long it, unsigned long long lpx)
+{
+    if (lane < f.parked) {
+        finish_parked<COUNT, BATCH>(a, w.park_s[lane], w.park_u[lane], BATCH ? w.park_f[lane] : 0u, it);
+        if (COUNT)
+            ++lpx;
+    }
+    if (COUNT) {
+        it = warp_sum_u64(it);
+        lpx = warp_sum_u64(lpx);
+        if (lane == 0) {
+            if (it) {
+                atomicAdd(&a.ctr->iterations, it);
+                atomicAdd(&a.ctr->leaf_iters, it);
+            }
+            if (lpx)
+                atomicAdd(&a.ctr->leaf_pixels, lpx);
+        }
+    }
+}
+
 }  // namespace ask
