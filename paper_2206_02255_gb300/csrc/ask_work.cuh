@@ -438,10 +438,13 @@ __device__ __forceinline__ void leaf_extent(DevCounters *ctr, uint32_t cap, uint
 // many or a band of the largest leaf would hold fewer than kLeafItemMinPx
 // pixels, one pre-pass: with whole leaves as items a map of few large leaves
 // kept most warps idle (n = 1024, g=16 r=2 B=32: 549 leaves of 32 x 32 for
-// 6080 warps; leaf kernel 219 -> 38 us).  A leaf of 65536 x 65536 pixels is
-// cut in two, so that an item's pixel count fits 32 bits.
-constexpr uint32_t kLeafItemsPerWarp = 4;
-constexpr uint32_t kLeafItemMinPx = 32;
+// 4864 warps; leaf kernel 219 -> 31 us), and a list of a few heavy leaves a
+// warp ended unevenly (n = 4096, 16 x 16 leaves: 356 us with 4 items a warp,
+// 337 with 8).  Bands of 32 pixels only halve the pre-passes' lanes (n = 1024:
+// 60 us against 54).  A leaf of 65536 x 65536 pixels is cut in two, so that an
+// item's pixel count fits 32 bits.
+constexpr uint32_t kLeafItemsPerWarp = 8;
+constexpr uint32_t kLeafItemMinPx = 64;
 __device__ __forceinline__ uint32_t leaf_item_shift(uint32_t leaves, uint32_t side, uint32_t warps)
 {
     const unsigned long long px = (unsigned long long)side * side;
