@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(1024) cdp2_pixel_kernel(CdpArgs a, Region g)
     unsigned long long it = 0;
     if (px < g.x0 + g.w && py < g.y0 + g.h && !on_perimeter(g, px, py)) {
         const float2 c = pixel_c(a.pm, px, py);
-        const uint32_t d = dwell(c.x, c.y, a.max_dwell);
+        const uint32_t d = dwell<false>(c.x, c.y, a.max_dwell);
         a.map[(size_t)py * a.n + px] = d;
         it = d;
     }
@@ -117,7 +117,7 @@ __device__ __forceinline__ void cdp2_region(const CdpArgs &a, const Region &g, u
             uint32_t px, py;
             perimeter_pixel(g, k, px, py);
             const float2 c = pixel_c(a.pm, px, py);
-            const uint32_t d = dwell(c.x, c.y, a.max_dwell);
+            const uint32_t d = dwell<false>(c.x, c.y, a.max_dwell);
             dmin = min(dmin, d);
             dmax = max(dmax, d);
             if (k < stage_cap)

@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(1024) leaf_kernel(LeafArgs a, uint32_t leaf_ca
         const uint32_t py = g.y0 + ty * blockDim.y + threadIdx.y;
         if (px < g.x0 + g.w && py < g.y0 + g.h && !(a.skip_perimeter && on_perimeter(g, px, py))) {
             const float2 c = pixel_c(a.pm, px, py);
-            const uint32_t d = dwell(c.x, c.y, a.max_dwell);
+            const uint32_t d = dwell<false>(c.x, c.y, a.max_dwell);
             a.map[(size_t)py * a.n + px] = d;
             if (COUNT) {
                 it += d;

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(1024) region_leaf_kernel(LeafArgs a)
                 const uint32_t px = g.x0 + tx0 + threadIdx.x, py = g.y0 + ty0 + threadIdx.y;
                 if (px < g.x0 + g.w && py < g.y0 + g.h) {
                     const float2 c = pixel_c(a.pm, px, py);
-                    const uint32_t d = dwell(c.x, c.y, a.max_dwell);
+                    const uint32_t d = dwell<false>(c.x, c.y, a.max_dwell);
                     a.map[(size_t)py * a.n + px] = d;
                     if (COUNT) {
                         it += d;
