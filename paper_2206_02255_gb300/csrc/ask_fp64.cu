@@ -69,8 +69,8 @@ __device__ __forceinline__ double2 pixel_c64(const PixelMap64 &pm, uint32_t px, 
 struct ArithF64 {
     using T = double;
     // Updates per unchecked block of the queries' and the leaf kernel's rounds
-    // (the test after each is 2 instructions of the FP64 pipe beside the
-    // block's 64: 8 updates took 9.36 ms on the map below, 16 9.11).
+    // (8 updates took 9.36 ms on the map below, 16 9.11; those and the figures
+    // by CTAs with x + x and the whole test on the FP64 pipe).
     static constexpr uint32_t kRound = 16;
     // CTAs an SM.  A warp instruction holds the SM's FP64 pipe for 16 cycles
     // however few lanes take part, and 2 warps a scheduler keep it busy, so
@@ -487,6 +487,17 @@ struct ParkW {
     uint32_t d[kLeaf64Warps][kPark64], pix[kLeaf64Warps][kPark64];
 };
 
+// The next pixels of a warp's band, up to 32: their points are computed by all
+// lanes at once and taken from here as lanes fall idle, one or two at a time.
+// Computed by the lanes that needed them, they cost every refill a 64-bit
+// division and (float-float) a dozen FP64 instructions: n = 1024 in seahorse
+// valley 6.42 -> 6.27 ms, n = 3000 on the antenna 7.46 -> 7.29 (float-float).
+template <class A>
+struct FreshW {
+    typename A::T cr[kLeaf64Warps][32], ci[kLeaf64Warps][32];
+    uint32_t pix[kLeaf64Warps][32];
+};
+
 template <class A, bool COUNT>
 __device__ __forceinline__ void resolve_parked_w(const Leaf64Args &a, ParkW<A> &pk, uint32_t wid,
                                                  uint32_t e, unsigned long long &it,
@@ -522,17 +533,20 @@ template <class A, bool COUNT>
 __global__ void __launch_bounds__(kLeaf64Warps * 32) leaf64_kernel(Leaf64Args a)
 {
     __shared__ ParkW<A> pk;
+    __shared__ FreshW<A> fresh;
     const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
     const uint32_t nleaves = min(a.ctr->leaf_count, a.leaf_cap);
     const uint32_t shift = leaf_item_shift64(nleaves, a.side, gridDim.x * kLeaf64Warps);
-    // warp-uniform: the leaf being handed out and how many of its pixels are
+    // warp-uniform: the band being handed out and how many of its pixels are
+    // (a leaf of 2^32 pixels is the only one, and cut), and the fresh points
+    // not yet taken
     Region cur;
     cur.x0 = cur.y0 = 0;
     cur.w = cur.h = 1;
-    unsigned long long next = 0, npix = 0;  // a leaf may hold up to 2^32 pixels
-    bool have = false, exhausted = false;
+    uint32_t next = 0, npix = 0, fresh_h = 0, fresh_n = 0;
     uint32_t parked = 0;
+    bool exhausted = false;
     // per lane: its orbit and pixel (x | y << 16; n <= 65536)
     OrbitW<A> o = orbit_w_start<A>(make_double2(0.0, 0.0));
     uint32_t pix = 0;
@@ -540,43 +554,56 @@ __global__ void __launch_bounds__(kLeaf64Warps * 32) leaf64_kernel(Leaf64Args a)
     unsigned long long it = 0, npx = 0;
     for (;;) {
         unsigned need = __ballot_sync(kAll, !busy);
-        while (need != 0u && !exhausted) {
-            if (!have) {
-                uint32_t li = 0;
-                if (lane == 0u)
-                    li = atomicAdd(&a.ctr->leaf_work, 1u);
-                li = __shfl_sync(kAll, li, 0);
-                if ((li >> shift) >= nleaves) {
-                    exhausted = true;
-                    break;
+        while (need != 0u && (fresh_n != 0u || !exhausted)) {
+            if (fresh_n == 0u) {
+                if (next >= npix) {
+                    uint32_t li = 0;
+                    if (lane == 0u)
+                        li = atomicAdd(&a.ctr->leaf_work, 1u);
+                    li = __shfl_sync(kAll, li, 0);
+                    if ((li >> shift) >= nleaves) {
+                        exhausted = true;
+                        break;
+                    }
+                    cur = unpack_region(a.leaves[li >> shift]);
+                    // rows [r0, r1) of the leaf
+                    const uint32_t band = li & ((1u << shift) - 1u);
+                    const uint32_t r0 = (uint32_t)(((unsigned long long)cur.h * band) >> shift);
+                    const uint32_t r1 = (uint32_t)(((unsigned long long)cur.h * (band + 1u)) >> shift);
+                    cur.y0 += r0;
+                    next = 0;
+                    npix = cur.w * (r1 - r0);
+                    if (npix == 0u)
+                        continue;
                 }
-                cur = unpack_region(a.leaves[li >> shift]);
-                // rows [r0, r1) of the leaf
-                const uint32_t band = li & ((1u << shift) - 1u);
-                const uint32_t r0 = (uint32_t)(((unsigned long long)cur.h * band) >> shift);
-                const uint32_t r1 = (uint32_t)(((unsigned long long)cur.h * (band + 1u)) >> shift);
-                if (r0 == r1)
-                    continue;
-                cur.y0 += r0;
-                cur.h = r1 - r0;
-                next = 0;
-                npix = (unsigned long long)cur.w * cur.h;
-                have = true;
+                __syncwarp();  // the points before have been read
+                fresh_h = 0;
+                fresh_n = min(32u, npix - next);
+                if (lane < fresh_n) {
+                    const uint32_t k = next + lane, ry = k / cur.w;
+                    const uint32_t px = cur.x0 + (k - ry * cur.w), py = cur.y0 + ry;
+                    const double2 c = pixel_c64(a.pm, px, py);
+                    fresh.cr[wid][lane] = A::from_double(c.x);
+                    fresh.ci[wid][lane] = A::from_double(c.y);
+                    fresh.pix[wid][lane] = px | (py << 16);
+                }
+                next += fresh_n;
+                __syncwarp();
             }
-            const unsigned long long avail = npix - next;
             const uint32_t rank = (uint32_t)__popc(need & below);
-            if (!busy && rank < avail) {
-                const unsigned long long k = next + rank;
-                const uint32_t ry = (uint32_t)(k / cur.w);
-                const uint32_t px = cur.x0 + (uint32_t)(k - (unsigned long long)ry * cur.w);
-                const uint32_t py = cur.y0 + ry;
-                o = orbit_w_start<A>(pixel_c64(a.pm, px, py));
-                pix = px | (py << 16);
+            if (!busy && rank < fresh_n) {
+                const uint32_t e = fresh_h + rank;
+                o.x = o.y = A::from_double(0.0);
+                o.cr = fresh.cr[wid][e];
+                o.ci = fresh.ci[wid][e];
+                o.d = 0;
+                o.fast = A::absorbing(o.cr, o.ci);
+                pix = fresh.pix[wid][e];
                 busy = true;
             }
-            next += min((unsigned long long)__popc(need), avail);
-            if (next >= npix)
-                have = false;
+            const uint32_t taken = min((uint32_t)__popc(need), fresh_n);
+            fresh_h += taken;
+            fresh_n -= taken;
             need = __ballot_sync(kAll, !busy);
         }
         if (__ballot_sync(kAll, busy) == 0u)
