@@ -952,9 +952,9 @@ def run_serve(args):
 # ---------------------------------------------------------------------------
 # Deep zoom: one double-precision map per step
 # ---------------------------------------------------------------------------
-# FP64-pipe operations per update in ask_fp64.cu: 3 DFMA + 1 DADD (the |z|^2
-# test is amortised over a block of updates)
-FP64_OPS_PER_ITER = 4
+# FP64-pipe operations per update in ask_fp64.cu: 3 DFMA (the doubling runs on
+# the integer pipe, the test mostly in single precision)
+FP64_OPS_PER_ITER = 3
 # Nominal FP64 rate of the GB300 table (1.25 TFLOP/s with an FMA as 2 flops):
 # 625 G FP64-pipe lane operations per second.  No measured FP64 peak exists.
 FP64_PEAK_GOPS = 1.25e3 / 2
