@@ -17,7 +17,7 @@
 // GB300 issues double-precision instructions at 1/64 of its single-precision
 // rate, so the binary64 kernels are bound by the FP64 pipe, and votes,
 // shared-memory parking and address arithmetic hide behind it; float-float
-// spends about 14x more instructions per update on a pipe 64x faster.  In
+// spends about 19x more instructions per update on a pipe 64x faster.  In
 // both, what matters is that lanes spend their arithmetic on useful updates:
 //  * level kernel: persistent, one warp per region from an atomic counter;
 //    the perimeter is queried 32 pixels at a time with the orbits in
