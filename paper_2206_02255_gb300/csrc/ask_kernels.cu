@@ -909,15 +909,16 @@ cudaError_t launch_init(uint2 *olt0, uint4 *rst0, DevCounters *ctr, uint32_t n, 
 {
     const uint32_t total = axis0 * rows;
     if (order != nullptr && olt0 != nullptr && total <= kInitOrderMax) {
-        return launch_chained(init_kernel, 1, 1024, 0, s, olt0, rst0, ctr, n, s0, axis0, row0, rows, *order, 1u);
+        init_kernel<<<1, 1024, 0, s>>>(olt0, rst0, ctr, n, s0, axis0, row0, rows, *order, 1u);
+        return cudaGetLastError();
     }
     uint32_t blocks = (total + 255u) / 256u;
     if (blocks < 1)
         blocks = 1;
     if (blocks > 4096)
         blocks = 4096;
-    return launch_chained(init_kernel, (int)blocks, 256, 0, s, olt0, rst0, ctr, n, s0, axis0, row0, rows,
-                          PixelMap{}, 0u);
+    init_kernel<<<blocks, 256, 0, s>>>(olt0, rst0, ctr, n, s0, axis0, row0, rows, PixelMap{}, 0u);
+    return cudaGetLastError();
 }
 
 template <bool COUNT, bool BATCH, int NS, bool PROVE>
@@ -973,7 +974,8 @@ cudaError_t launch_fill(const FillArgs &f, bool batch, int sms, cudaStream_t s)
 cudaError_t launch_init_batch(uint4 *olt0, uint4 *rst0, DevCounters *ctr, const FrameDesc *frames,
                               uint32_t nframes, uint32_t total0, cudaStream_t s)
 {
-    return launch_chained(init_batch_kernel, (int)nframes, 256, 0, s, olt0, rst0, ctr, frames, total0);
+    init_batch_kernel<<<nframes, 256, 0, s>>>(olt0, rst0, ctr, frames, total0);
+    return cudaGetLastError();
 }
 
 template <bool COUNT, bool BATCH>

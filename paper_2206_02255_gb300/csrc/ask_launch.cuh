@@ -1,14 +1,20 @@
 // ask_launch.cuh -- launches of the ASK chain's kernels.
 //
-// Every kernel of a chain (init, levels, leaves) is launched as a programmatic
-// dependent of the kernel before it on the stream, says at its start that its
-// own dependent may be launched (chain_start), and waits there for the kernels
-// before it to finish before it touches memory.  So a kernel's launch and the
-// set-up of its CTAs overlap the end of the one before; what it reads and
-// writes is ordered as in plain stream order, since the wait covers the whole
-// earlier grid and its memory operations, and that grid has itself waited for
-// the one before it.  n = 256: 56 -> 49 us; n = 1024: 79 -> 71 us; n = 16384:
-// 1625 -> 1614 us.
+// The kernels of a chain after its first (init, plainly launched; then levels
+// and leaves) are launched as programmatic dependents of the kernel before
+// them on the stream: each says at its start that its own dependent may be
+// launched (chain_start), and waits there for the kernels before it to finish
+// before it touches memory.  So a kernel's launch and the set-up of its CTAs
+// overlap the end of the one before; what it reads and writes is ordered as in
+// plain stream order, since the wait covers the whole earlier grid and its
+// memory operations, and that grid has itself waited for the one before it.
+// n = 256: 56 -> 49 us; n = 1024: 79 -> 71 us; n = 16384: 1625 -> 1614 us.
+//
+// The init kernel depends on whatever the stream held before: a CDP2 render of
+// the same scratch, say, whose grids launch the rest of their work from the
+// device.  The wait is defined for the grid before, not for the grids that it
+// has launched in its turn, so init takes plain stream order, which covers
+// those.
 //
 // The deep-zoom kernels are launched plainly: their grids leave room on an SM,
 // and CTAs placed while the kernel before still holds a part of the SMs end
