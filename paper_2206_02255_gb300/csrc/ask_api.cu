@@ -745,8 +745,8 @@ struct BatchPlan {
     uint32_t leaf_side = 0;               // largest nominal leaf side over the frames
     uint64_t pixels = 0;                  // of all frames
     // the persistent batch kernel: queue items (every level's chunk items and
-    // fill bands of every frame), chunk states, level-0 items and states
-    uint64_t q_items = 0, q_states = 0, q_total0 = 0, q_states0 = 0;
+    // fill bands of every frame), chunk states, level-0 items and states, leaf-list entries
+    uint64_t q_items = 0, q_states = 0, q_total0 = 0, q_states0 = 0, q_leaves = 0;
 };
 
 // Chunk items per region of a level of side s in the persistent batch
@@ -819,9 +819,11 @@ ask_status plan_batch(ask_ctx *ctx, const ask_frame *frames, uint32_t nframes, u
         bp.q_total0 += regions0 * d.chunks[0];
         if (d.chunks[0] > 1u)
             bp.q_states0 += regions0;
+        const uint32_t leaf_side = plan.side[plan.levels - 1];
         bp.leaf_need += plan.max_regions[plan.levels - 1];
+        bp.q_leaves += plan.max_regions[plan.levels - 1] * queue_leaf_bands(leaf_side, leaf_side);
         bp.pixels += (uint64_t)fr.n * fr.n;
-        bp.leaf_side = std::max(bp.leaf_side, plan.side[plan.levels - 1]);
+        bp.leaf_side = std::max(bp.leaf_side, leaf_side);
         total0 += (uint64_t)plan.axis0 * plan.axis0;
         if (plan.levels > bp.L)
             bp.L = plan.levels;
@@ -844,7 +846,8 @@ ask_status plan_batch(ask_ctx *ctx, const ask_frame *frames, uint32_t nframes, u
     }
     if (bp.leaf_need >= 0xffffffffull || bp.fill_need >= 0xffffffffull)
         return set_err(ctx, ASK_EINVAL, "batch too large");
-    if ((flags & ASK_FLAG_PERSISTENT) && (bp.q_items >= 0xffffffffull || bp.q_states >= 0xffffffffull))
+    if ((flags & ASK_FLAG_PERSISTENT) && (bp.q_items >= 0xffffffffull || bp.q_states >= 0xffffffffull ||
+                                          bp.q_leaves >= 0xffffffffull))
         return set_err(ctx, ASK_EINVAL, "batch too large for the persistent kernel's work queue");
     bp.total0 = (uint32_t)total0;
     return ASK_OK;
@@ -1038,7 +1041,7 @@ ask_status reserve_queue(ask_ctx *ctx, QueueBuffers &b, const BatchPlan &bp, boo
     if ((st = grow(ctx, &b.rst, &b.rst_cap, std::max<uint64_t>(bp.q_states, 1), "cudaMalloc(query states)")) !=
         ASK_OK)
         return st;
-    if ((st = grow_zeroed(ctx, &b.leaves, &b.leaf_cap, bp.leaf_need, "cudaMalloc(leaf list)")) != ASK_OK)
+    if ((st = grow_zeroed(ctx, &b.leaves, &b.leaf_cap, bp.q_leaves, "cudaMalloc(leaf list)")) != ASK_OK)
         return st;
     if ((st = grow(ctx, &b.frames, &b.frames_cap, (uint64_t)bp.desc.size(), "cudaMalloc(frame table)")) != ASK_OK)
         return st;

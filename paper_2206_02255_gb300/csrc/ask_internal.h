@@ -37,7 +37,8 @@ struct DevCounters {
     uint32_t pool_count;                    // survivors put in the pool (may exceed its capacity)
     uint32_t pool_work;                     // next pool entries handed out
     uint32_t leaf_light;                    // leaf-list entries from the back (level kernels:
-                                            // leaves whose probe escaped, taken last)
+                                            // leaves whose probe escaped, taken last; persistent
+                                            // kernel: minus the entries of leaves beyond one each)
     uint32_t back[ASK_MAX_LEVELS + 1];      // region-table entries of level i written from the
                                             // back (count[i] holds those from the front)
 };
@@ -236,7 +237,7 @@ struct QueueArgs {
     uint32_t item_cap;
     uint4 *rst;           // chunk-query states {common dwell, differs, chunks done, -}
     uint32_t rst_cap;
-    uint4 *leaves;        // leaf list {origin, extent, frame, epoch}
+    uint4 *leaves;        // leaf list {origin, extent, frame, epoch}: leaves, or bands of large ones
     uint32_t leaf_cap;
     const FrameDesc *frames;
     DevCounters *ctr;
@@ -251,6 +252,17 @@ struct QueueArgs {
 // chunks; the tag has 6 bits for the chunk).
 constexpr uint32_t kChunkPxQueue = 128;
 constexpr uint32_t kMaxChunksQueue = 16;
+// A leaf of more than kQueueLeafPx pixels goes to the leaf list as bands of
+// whole rows, at most that many pixels each: a warp takes whole entries and
+// counts their pixels in 32 bits, which those of a leaf of 65536 x 65536 do not
+// fit.
+constexpr uint32_t kQueueLeafPx = 1u << 20;
+__host__ __device__ inline uint32_t queue_leaf_rows(uint32_t w) { return w >= kQueueLeafPx ? 1u : kQueueLeafPx / w; }
+__host__ __device__ inline uint32_t queue_leaf_bands(uint32_t w, uint32_t h)
+{
+    const uint32_t rows = queue_leaf_rows(w);
+    return h / rows + (h % rows != 0u);
+}
 // Idle polls in a row (with __nanosleep back-off of up to 256 ns, reset
 // whenever the queue or the leaf list moves) before a warp gives up.
 constexpr uint32_t kQueueWaitLimit = 1u << 26;

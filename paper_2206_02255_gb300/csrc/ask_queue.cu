@@ -280,18 +280,27 @@ __device__ __forceinline__ void process_item(const QueueArgs &q, uint32_t t, uin
         return;
     }
     if (!f.split) {
-        // a leaf: appended to the published leaf list
+        // a leaf: appended to the published leaf list (leaf_light takes the
+        // entries beyond one off the count of leaves, modulo 2^32)
+        const uint32_t nb = queue_leaf_bands(g.w, g.h), rows = queue_leaf_rows(g.w);
+        uint32_t slot = 0;
         if (lane == 0) {
-            const uint32_t slot = atomicAdd(&q.ctr->leaf_count, 1u);
-            if (slot < q.leaf_cap) {
-                uint4 *l = &q.leaves[slot];
-                l->x = e.x;
-                l->y = e.y;
-                l->z = frame;
-                store_release(&l->w, epoch);
-            } else {
+            slot = atomicAdd(&q.ctr->leaf_count, nb);
+            if (nb > 1u)
+                atomicSub(&q.ctr->leaf_light, nb - 1u);
+        }
+        slot = __shfl_sync(kFull, slot, 0);
+        for (uint32_t k = lane; k < nb; k += 32u) {
+            if (slot + k >= q.leaf_cap) {
                 atomicOr(&q.ctr->error, ERR_LEAF_OVERFLOW);
+                break;
             }
+            const uint2 band = pack_region(g.x0, g.y0 + k * rows, g.w, min(rows, g.h - k * rows));
+            uint4 *l = &q.leaves[slot + k];
+            l->x = band.x;
+            l->y = band.y;
+            l->z = frame;
+            store_release(&l->w, epoch);
         }
         finish_item(q, epoch, lane);
         return;
