@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
         if (decided) {
             uint32_t kind;
             if (uniform) {
-                const uint32_t area = g.w * g.h;
+                const unsigned long long area = (unsigned long long)g.w * g.h;
                 if (a.fills != nullptr && area > kInPlaceFillArea) {
                     kind = KIND_FILL_LATER;
                 } else {
@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(256, kLevelMinBlocks2) level_cta_kernel(LevelA
         const uint32_t wv = st.x;
         uint32_t kind = f.split ? KIND_SPLIT : KIND_LEAF;
         if (uniform) {
-            const uint32_t area = g.w * g.h;
+            const unsigned long long area = (unsigned long long)g.w * g.h;
             kind = (a.fills != nullptr && area > kInPlaceFillArea) ? KIND_FILL_LATER : KIND_FILL;
             if (kind == KIND_FILL)
                 fill_rect(f.map, f.n, g, wv, threadIdx.x, blockDim.x);

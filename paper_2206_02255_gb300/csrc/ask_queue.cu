@@ -255,7 +255,7 @@ __device__ __forceinline__ void process_item(const QueueArgs &q, uint32_t t, uin
     if (uniform) {
         if (lane == 0)
             atomicAdd(&q.ctr->fills[level], 1u);
-        const uint32_t area = g.w * g.h;
+        const unsigned long long area = (unsigned long long)g.w * g.h;
         if (area <= kInPlaceFillArea) {
             fill_rect(f.map, f.n, g, wv, lane, 32u);
             finish_item(q, epoch, lane);
