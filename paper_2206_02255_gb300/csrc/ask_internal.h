@@ -167,6 +167,21 @@ __host__ __device__ inline uint32_t fill_band_count(uint32_t w, uint32_t h)
 }
 cudaError_t launch_level(const LevelArgs &a, bool count, bool batch, int sms, cudaStream_t s);
 
+// Tickets of a level kernel: `heavy` of one item each, then the `light` items
+// `take` at a time.
+__host__ __device__ inline uint32_t level_tickets(uint32_t heavy, uint32_t light, uint32_t take)
+{
+    return heavy + light / take + (light % take != 0u);
+}
+// Whether the ticket that a warp got from the counter, `warps` + its value, lies
+// past the last one.  Every warp asks once more after the last, so the sum may
+// wrap, by less than the number of warps; no valid ticket of the counter is
+// that small.
+__host__ __device__ inline bool past_tickets(uint32_t t, uint32_t warps, uint32_t tickets)
+{
+    return t >= tickets || t < warps;
+}
+
 struct FillArgs {
     uint32_t *map;        // single frame (batch entries name their frame)
     uint32_t n;
@@ -211,6 +226,34 @@ inline uint64_t pool_need(uint64_t pixels)
 {
     return pixels > kPoolPixels ? 0u : pixels < kPoolEntries ? pixels : kPoolEntries;
 }
+// How finely leaves are handed out: 1 << shift row bands per leaf.  A list
+// with fewer than kLeafItemsPerWarp items a warp is cut until it has that
+// many or a band of the largest leaf would hold fewer than kLeafItemMinPx
+// pixels, one pre-pass: with whole leaves as items a map of few large leaves
+// kept most warps idle (n = 1024, g=16 r=2 B=32: 549 leaves of 32 x 32 for
+// 4864 warps; leaf kernel 219 -> 31 us), and a list of a few heavy leaves a
+// warp ended unevenly (n = 4096, 16 x 16 leaves: 356 us with 4 items a warp,
+// 337 with 8).  Bands of 32 pixels only halve the pre-passes' lanes (n = 1024:
+// 60 us against 54).  A leaf of 65536 x 65536 pixels is cut in two, so that an
+// item's pixel count fits 32 bits.
+constexpr uint32_t kLeafItemsPerWarp = 8;
+constexpr uint32_t kLeafItemMinPx = 64;
+__host__ __device__ inline uint32_t leaf_item_shift(uint32_t leaves, uint32_t side, uint32_t warps)
+{
+    const unsigned long long px = (unsigned long long)side * side;
+    uint32_t shift = side > 65535u ? 1u : 0u;
+    while (((unsigned long long)leaves << shift) < (unsigned long long)kLeafItemsPerWarp * warps &&
+           (px >> (shift + 1u)) >= kLeafItemMinPx && (2u << shift) <= side)
+        ++shift;
+    return shift;
+}
+// Whether a 32-bit counter can hand out the items: every warp asks once more
+// after the last (2^31 leaves cut in two would wrap, and never run out).
+__host__ __device__ inline bool leaf_items_fit(uint32_t leaves, uint32_t shift, uint32_t warps)
+{
+    return ((unsigned long long)leaves << shift) + warps <= 0xffffffffull;
+}
+
 // tiled = false: lane-refill kernel (default); true: one thread per pixel in
 // block_x x block_y tiles (single frame only)
 cudaError_t launch_leaf(const LeafArgs &a, uint32_t bx, uint32_t by, bool count, bool tiled,

@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
     uint32_t take = 1u;
     while (take < kTicketMax && light / (2u * take) >= kTicketsPerWarp * warps)
         take *= 2u;
-    const uint32_t tickets = heavy + (light + take - 1u) / take;
+    const uint32_t tickets = level_tickets(heavy, light, take);
     uint32_t todo = 0, my_c = 0, my_slot = 0;
     T mine = T();
     // a warp's first ticket is its number (counted over the CTAs first, so that
@@ -455,9 +455,9 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
                     t = warps + atomicAdd(&a.ctr->work[a.level], 1u);
                 t = __shfl_sync(kFull, t, 0);
             }
-            fresh = false;
-            if (t >= tickets)
+            if (fresh ? t >= tickets : past_tickets(t, warps, tickets))
                 break;
+            fresh = false;
             // lane k looks at the ticket's k-th item: its record, and, of a
             // large region, whether it is still open
             bool open;
@@ -789,8 +789,13 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocks) leaf_refi
     if (threadIdx.x == 0) {
         uint32_t front, total;
         leaf_extent(a.ctr, a.leaf_cap, front, total);
-        extent = make_uint3(front, total,
-                            leaf_item_shift(total, a.side, gridDim.x * (uint32_t)kRefillWarps));
+        const uint32_t warps = gridDim.x * (uint32_t)kRefillWarps;
+        const uint32_t shift = leaf_item_shift(total, a.side, warps);
+        if (!leaf_items_fit(total, shift, warps)) {
+            atomicOr(&a.ctr->error, ERR_LEAF_OVERFLOW);
+            total = 0;
+        }
+        extent = make_uint3(front, total, shift);
     }
     __syncthreads();
     if (a.fills != nullptr && wib == kRefillWarps - 1u)

@@ -433,28 +433,6 @@ __device__ __forceinline__ void leaf_extent(DevCounters *ctr, uint32_t cap, uint
         atomicOr(&ctr->error, ERR_LEAF_OVERFLOW);
 }
 
-// How finely leaves are handed out: 1 << shift row bands per leaf.  A list
-// with fewer than kLeafItemsPerWarp items a warp is cut until it has that
-// many or a band of the largest leaf would hold fewer than kLeafItemMinPx
-// pixels, one pre-pass: with whole leaves as items a map of few large leaves
-// kept most warps idle (n = 1024, g=16 r=2 B=32: 549 leaves of 32 x 32 for
-// 4864 warps; leaf kernel 219 -> 31 us), and a list of a few heavy leaves a
-// warp ended unevenly (n = 4096, 16 x 16 leaves: 356 us with 4 items a warp,
-// 337 with 8).  Bands of 32 pixels only halve the pre-passes' lanes (n = 1024:
-// 60 us against 54).  A leaf of 65536 x 65536 pixels is cut in two, so that an
-// item's pixel count fits 32 bits.
-constexpr uint32_t kLeafItemsPerWarp = 8;
-constexpr uint32_t kLeafItemMinPx = 64;
-__device__ __forceinline__ uint32_t leaf_item_shift(uint32_t leaves, uint32_t side, uint32_t warps)
-{
-    const unsigned long long px = (unsigned long long)side * side;
-    uint32_t shift = side > 65535u ? 1u : 0u;
-    while (((unsigned long long)leaves << shift) < (unsigned long long)kLeafItemsPerWarp * warps &&
-           (px >> (shift + 1u)) >= kLeafItemMinPx && (2u << shift) <= side)
-        ++shift;
-    return shift;
-}
-
 // The leaf list of a launch chain: complete when the leaf kernel starts, its
 // leaves (or row bands of them, see leaf_item_shift) handed out one at a time
 // by a device counter.

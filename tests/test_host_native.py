@@ -18,7 +18,7 @@ def checks(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("name", ["queue_leaf_entries"])
+@pytest.mark.parametrize("name", ["queue_leaf_entries", "level_ticket_counter", "leaf_item_counter"])
 def test_host_rule(checks, name):
     r = subprocess.run([checks, name], stdout=subprocess.PIPE, text=True)
     assert r.returncode == 0, r.stdout
