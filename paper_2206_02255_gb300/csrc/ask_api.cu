@@ -28,6 +28,7 @@ struct BatchBuffers {
     uint64_t pool_cap = 0;
     uint32_t *pool_f = nullptr;
     uint64_t pool_f_cap = 0;
+    uint64_t pool_refused = ~0ull;       // entries that did not fit the device's memory
     ask::FrameDesc *frames = nullptr;    // device frame table
     uint64_t frames_cap = 0;
     ask::DevCounters *ctr = nullptr;     // not owned when it is the context's
@@ -853,6 +854,25 @@ ask_status plan_batch(ask_ctx *ctx, const ask_frame *frames, uint32_t nframes, u
     return ASK_OK;
 }
 
+// The survivor pool, last of a batch's scratch and the only part that it can
+// do without: where the device has no memory left for it, the leaf kernel's
+// warps keep their survivors (and the same size is not tried again).
+void reserve_pool(BatchBuffers &b, uint64_t need)
+{
+    if (need >= b.pool_refused)
+        return;
+    if (grow((ask_ctx *)nullptr, &b.pool, &b.pool_cap, need, "") == ASK_OK &&
+        grow((ask_ctx *)nullptr, &b.pool_f, &b.pool_f_cap, need, "") == ASK_OK)
+        return;
+    cudaGetLastError();  // a refused allocation is not sticky
+    cudaFree(b.pool);
+    cudaFree(b.pool_f);
+    b.pool = nullptr;
+    b.pool_f = nullptr;
+    b.pool_cap = b.pool_f_cap = 0;
+    b.pool_refused = need;
+}
+
 ask_status reserve_batch(ask_ctx *ctx, BatchBuffers &b, const BatchPlan &bp, bool own_counters)
 {
     ask_status st;
@@ -878,10 +898,6 @@ ask_status reserve_batch(ask_ctx *ctx, BatchBuffers &b, const BatchPlan &bp, boo
         return st;
     if ((st = grow(ctx, &b.fills, &b.fill_cap, bp.fill_need, "cudaMalloc(batch fills)")) != ASK_OK)
         return st;
-    const uint64_t pool = pool_need(bp.pixels);
-    if ((st = grow(ctx, &b.pool, &b.pool_cap, pool, "cudaMalloc(survivor pool)")) != ASK_OK ||
-        (st = grow(ctx, &b.pool_f, &b.pool_f_cap, pool, "cudaMalloc(survivor pool)")) != ASK_OK)
-        return st;
     if ((st = grow(ctx, &b.frames, &b.frames_cap, (uint64_t)bp.desc.size(), "cudaMalloc(frame table)")) !=
         ASK_OK)
         return st;
@@ -892,6 +908,7 @@ ask_status reserve_batch(ask_ctx *ctx, BatchBuffers &b, const BatchPlan &bp, boo
         if (e != cudaSuccess)
             return cuda_err(ctx, e, "cudaMalloc(batch counters)");
     }
+    reserve_pool(b, pool_need(bp.pixels));
     return ASK_OK;
 }
 
@@ -967,7 +984,8 @@ ask_status enqueue_batch(ask_ctx *ctx, const BatchBuffers &b, const BatchPlan &b
     la.bound = bp.leaf_need;
     la.side = bp.leaf_side;
     la.skip_perimeter = exact ? 1u : 0u;
-    const uint64_t pool = pool_need(bp.pixels);
+    const uint64_t need = pool_need(bp.pixels);
+    const uint64_t pool = (b.pool_cap >= need && b.pool_f_cap >= need) ? need : 0u;
     la.pool = pool ? b.pool : nullptr;
     la.pool_frame = pool ? b.pool_f : nullptr;
     la.pool_cap = (uint32_t)pool;

@@ -1,11 +1,75 @@
 // Checks of the library's host-side rules that need no GPU: one check per
 // name on the command line; a failed one prints its line and exits with 1.
+//
+// The host driver is compiled in with a CUDA runtime of our own in the place
+// of the calls below, and with launches that do nothing but record.
+#include <cuda_runtime.h>
+
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 
-#include "ask_internal.h"
+static size_t g_malloc_limit = ~(size_t)0;  // a larger allocation fails
+static size_t g_malloc_refused = 0;         // and one of this size
+static int g_malloc_failed = 0;
+static cudaError_t g_last = cudaSuccess;
 
-using namespace ask;
+template <typename T>
+static cudaError_t fake_malloc(T **p, size_t bytes)
+{
+    if (bytes > g_malloc_limit || bytes == g_malloc_refused) {
+        ++g_malloc_failed;
+        return g_last = cudaErrorMemoryAllocation;
+    }
+    *p = static_cast<T *>(std::malloc(bytes < 64 ? bytes : 64));  // never touched
+    return cudaSuccess;
+}
+static cudaError_t fake_free(void *p)
+{
+    std::free(p);
+    return cudaSuccess;
+}
+static cudaError_t fake_memset(void *, int, size_t) { return cudaSuccess; }
+static cudaError_t fake_get_last_error()
+{
+    const cudaError_t e = g_last;
+    g_last = cudaSuccess;
+    return e;
+}
+#define cudaMalloc fake_malloc
+#define cudaFree fake_free
+#define cudaMemset fake_memset
+#define cudaGetLastError fake_get_last_error
+
+#include "ask_api.cu"
+
+namespace ask {
+static LeafArgs g_leaf;  // of the last leaf launch
+#define RECORDS_NOTHING(name, ...) \
+    cudaError_t name(__VA_ARGS__) { return cudaSuccess; }
+RECORDS_NOTHING(launch_exhaustive, uint32_t *, uint32_t, PixelMap, uint32_t, uint32_t, uint32_t, bool,
+                DevCounters *, cudaStream_t)
+RECORDS_NOTHING(launch_init, uint2 *, uint4 *, DevCounters *, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t,
+                cudaStream_t, const PixelMap *)
+RECORDS_NOTHING(launch_init_batch, uint4 *, uint4 *, DevCounters *, const FrameDesc *, uint32_t, uint32_t,
+                cudaStream_t)
+RECORDS_NOTHING(launch_level, const LevelArgs &, bool, bool, int, cudaStream_t)
+RECORDS_NOTHING(launch_fill, const FillArgs &, bool, int, cudaStream_t)
+RECORDS_NOTHING(launch_queue, const QueueArgs &, uint32_t, bool, int, cudaStream_t)
+RECORDS_NOTHING(launch_cdp2, const CdpArgs &, uint32_t, uint32_t, uint32_t, uint32_t, cudaStream_t)
+RECORDS_NOTHING(cdp2_set_pending_limit, size_t)
+RECORDS_NOTHING(launch_level_region, const LevelArgs &, bool, bool, uint32_t, int, cudaStream_t)
+RECORDS_NOTHING(launch_leaf_region, const LeafArgs &, uint32_t, uint32_t, bool, int, cudaStream_t)
+RECORDS_NOTHING(launch_exhaustive64, uint32_t *, uint32_t, PixelMap64, uint32_t, uint32_t, uint32_t, bool, bool,
+                DevCounters *, cudaStream_t)
+RECORDS_NOTHING(launch_level64, const Level64Args &, bool, bool, int, cudaStream_t)
+RECORDS_NOTHING(launch_leaf64, const Leaf64Args &, bool, bool, int, cudaStream_t)
+cudaError_t launch_leaf(const LeafArgs &a, uint32_t, uint32_t, bool, bool, bool, int, cudaStream_t)
+{
+    g_leaf = a;
+    return cudaSuccess;
+}
+}  // namespace ask
 
 #define EXPECT(c)                                                   \
     do {                                                            \
@@ -77,6 +141,49 @@ static int leaf_item_counter()
     return 0;
 }
 
+// A small batch on a device with no memory left for its survivor pool renders
+// without one, and with one once a smaller batch's fits.
+static int pool_does_not_fit()
+{
+    alignas(16) static uint32_t map[4];
+    const ask_frame big = {{-1.5f, 0.5f, -1.0f, 1.0f}, 1500, 100, 8, 2, 32, 0, map};
+    const ask_frame small = {{-1.5f, 0.5f, -1.0f, 1.0f}, 300, 100, 2, 2, 32, 0, map};
+    ask_ctx ctx{};
+    ctx.dev.sms = 152;
+    BatchBuffers b;
+    BatchPlan bp, bq;
+    uint32_t launches = 0, with = 0;
+    EXPECT(plan_batch(&ctx, &big, 1, 0, 0, bp) == ASK_OK && pool_need(bp.pixels) == 1500u * 1500u);
+    EXPECT(plan_batch(&ctx, &small, 1, 0, 0, bq) == ASK_OK && pool_need(bq.pixels) == 300u * 300u);
+    for (size_t entry : {sizeof(float4), sizeof(uint32_t)}) {
+        g_malloc_refused = 1500 * 1500 * entry;
+        g_malloc_failed = 0;
+        for (int k = 0; k < 2; ++k) {  // the second call does not ask again
+            EXPECT(reserve_batch(&ctx, b, bp, true) == ASK_OK);
+            EXPECT(g_malloc_failed == 1 && g_last == cudaSuccess && ctx.err[0] == 0);
+            EXPECT(enqueue_batch(&ctx, b, bp, 0, nullptr, &launches) == ASK_OK);
+            EXPECT(g_leaf.pool == nullptr && g_leaf.pool_frame == nullptr && g_leaf.pool_cap == 0);
+        }
+        EXPECT(reserve_batch(&ctx, b, bq, true) == ASK_OK);
+        EXPECT(enqueue_batch(&ctx, b, bq, 0, nullptr, &with) == ASK_OK);
+        EXPECT(g_leaf.pool != nullptr && g_leaf.pool_frame != nullptr && g_leaf.pool_cap == 300u * 300u);
+        EXPECT(enqueue_batch(&ctx, b, bp, 0, nullptr, &launches) == ASK_OK && g_leaf.pool == nullptr);
+        free_batch(b, true);
+    }
+    g_malloc_refused = 0;
+    // memory that the batch cannot do without is an error as ever
+    g_malloc_limit = 64;
+    EXPECT(reserve_batch(&ctx, b, bp, true) == ASK_ENOMEM);
+    free_batch(b, true);
+    // with memory enough
+    g_malloc_limit = ~(size_t)0;
+    EXPECT(reserve_batch(&ctx, b, bp, true) == ASK_OK);
+    EXPECT(enqueue_batch(&ctx, b, bp, 0, nullptr, &with) == ASK_OK);
+    EXPECT(g_leaf.pool == b.pool && g_leaf.pool_cap == 1500u * 1500u && with == launches + 1u);
+    free_batch(b, true);
+    return 0;
+}
+
 struct Check {
     const char *name;
     int (*fn)();
@@ -85,6 +192,7 @@ static const Check kChecks[] = {
     {"queue_leaf_entries", queue_leaf_entries},
     {"level_ticket_counter", level_ticket_counter},
     {"leaf_item_counter", leaf_item_counter},
+    {"pool_does_not_fit", pool_does_not_fit},
 };
 
 int main(int argc, char **argv)

@@ -18,7 +18,8 @@ def checks(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("name", ["queue_leaf_entries", "level_ticket_counter", "leaf_item_counter"])
+@pytest.mark.parametrize("name", ["queue_leaf_entries", "level_ticket_counter", "leaf_item_counter",
+                                  "pool_does_not_fit"])
 def test_host_rule(checks, name):
     r = subprocess.run([checks, name], stdout=subprocess.PIPE, text=True)
     assert r.returncode == 0, r.stdout
