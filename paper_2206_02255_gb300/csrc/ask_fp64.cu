@@ -685,7 +685,8 @@ template <class A, bool COUNT>
 static cudaError_t level_w_launch(const Level64Args &a, int sms, cudaStream_t s)
 {
     const int threads = (int)kLevel64Warps * 32;
-    static const int resident = std::min(resident_ctas(level64_kernel<A, COUNT>, threads, 0), A::kLevelCtas);
+    static PerDevice known;
+    const int resident = std::min(resident_ctas(level64_kernel<A, COUNT>, threads, 0, &known), A::kLevelCtas);
     level64_kernel<A, COUNT><<<resident * sms, threads, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -701,7 +702,8 @@ template <class A, bool COUNT>
 static cudaError_t leaf_w_launch(const Leaf64Args &a, int sms, cudaStream_t s)
 {
     const int threads = (int)kLeaf64Warps * 32;
-    static const int resident = std::min(resident_ctas(leaf64_kernel<A, COUNT>, threads, 0), A::kLeafCtas);
+    static PerDevice known;
+    const int resident = std::min(resident_ctas(leaf64_kernel<A, COUNT>, threads, 0, &known), A::kLeafCtas);
     leaf64_kernel<A, COUNT><<<resident * sms, threads, 0, s>>>(a);
     return cudaGetLastError();
 }

@@ -931,13 +931,12 @@ static cudaError_t level_launch(const LevelArgs &a, int sms, cudaStream_t s)
 {
     const size_t stage = (size_t)(256 / 32) * kWarpStage * sizeof(uint32_t);
     const size_t smem = a.exact_last ? stage : 0u;
-    static const int plain = resident_ctas(level_kernel<COUNT, BATCH, NS, PROVE>, 256, 0);
-    static const int staged = resident_ctas(level_kernel<COUNT, BATCH, NS, PROVE>, 256, stage);
+    static PerDevice plain, staged;
     // no more CTAs than the level can have items for, but one an SM as long as
     // there is an item for each
     const unsigned long long items = a.bound * a.chunks;
     const unsigned long long most = std::max((items + 7u) / 8u, std::min(items, (unsigned long long)sms));
-    int grid = (a.exact_last ? staged : plain) * sms;
+    int grid = resident_ctas(level_kernel<COUNT, BATCH, NS, PROVE>, 256, smem, a.exact_last ? &staged : &plain) * sms;
     if (most < (unsigned long long)grid)
         grid = most ? (int)most : 1;
     return launch_chained(level_kernel<COUNT, BATCH, NS, PROVE>, grid, 256, smem, s, a);
@@ -989,12 +988,13 @@ static cudaError_t refill_launch(const LeafArgs &a, int sms, cudaStream_t s)
     const int threads = kRefillWarps * 32;
     // no more CTAs than the leaves can have pre-passes for
     const unsigned long long most = a.bound * a.side * a.side / (64u * kRefillWarps) + 1u;
-    static const int resident = resident_ctas(leaf_refill_kernel<COUNT, BATCH>, threads, 0);
+    static PerDevice known, known_pool;
+    const int resident = resident_ctas(leaf_refill_kernel<COUNT, BATCH>, threads, 0, &known);
     const int grid = (int)std::min<unsigned long long>(most, (unsigned long long)(resident * sms));
     const cudaError_t e = launch_chained(leaf_refill_kernel<COUNT, BATCH>, grid, threads, 0, s, a);
     if (!BATCH || e != cudaSuccess || a.pool == nullptr)
         return e;
-    static const int pooled = resident_ctas(pool_kernel<COUNT>, threads, 0);
+    const int pooled = resident_ctas(pool_kernel<COUNT>, threads, 0, &known_pool);
     const int pgrid = (int)std::min<unsigned long long>(most, (unsigned long long)(pooled * sms));
     return launch_chained(pool_kernel<COUNT>, pgrid, threads, 0, s, a, (uint32_t)pooled);
 }

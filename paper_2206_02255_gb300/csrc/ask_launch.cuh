@@ -23,6 +23,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <utility>
 
 namespace ask {
@@ -50,14 +51,28 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), int grid, int threads, size
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// CTAs of a kernel that fit an SM at once (at least 1).
+// Answers of resident_ctas, by device (0: not asked yet).
+constexpr int kKnownDevices = 64;
+struct PerDevice {
+    std::atomic<int> ctas[kKnownDevices] = {};
+};
+
+// CTAs of a kernel that fit an SM of the current device at once (at least 1).
+// `known` keeps the answer; a query that failed counts as 1 this once.
 template <typename K>
-int resident_ctas(K kernel, int threads, size_t smem)
+int resident_ctas(K kernel, int threads, size_t smem, PerDevice *known = nullptr)
 {
-    int per_sm = 0;
+    int dev = -1, per_sm = 0;
+    if (known && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kKnownDevices &&
+        (per_sm = known->ctas[dev].load(std::memory_order_relaxed)) > 0)
+        return per_sm;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
+        per_sm < 1) {
+        cudaGetLastError();  // not the launch's error
+        return 1;
+    }
+    if (known && dev >= 0 && dev < kKnownDevices)
+        known->ctas[dev].store(per_sm, std::memory_order_relaxed);
     return per_sm;
 }
 

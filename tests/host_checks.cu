@@ -36,12 +36,28 @@ static cudaError_t fake_get_last_error()
     g_last = cudaSuccess;
     return e;
 }
+static int g_device = 0, g_occupancy[100], g_occupancy_asked = 0;  // 0: the query fails
+static cudaError_t fake_get_device(int *d)
+{
+    *d = g_device;
+    return cudaSuccess;
+}
+template <typename K>
+static cudaError_t fake_occupancy(int *per_sm, K, int, size_t)
+{
+    ++g_occupancy_asked;
+    *per_sm = g_occupancy[g_device];
+    return *per_sm ? cudaSuccess : (g_last = cudaErrorInvalidDevice);
+}
+#define cudaGetDevice fake_get_device
+#define cudaOccupancyMaxActiveBlocksPerMultiprocessor fake_occupancy
 #define cudaMalloc fake_malloc
 #define cudaFree fake_free
 #define cudaMemset fake_memset
 #define cudaGetLastError fake_get_last_error
 
 #include "ask_api.cu"
+#include "ask_launch.cuh"
 
 namespace ask {
 static LeafArgs g_leaf;  // of the last leaf launch
@@ -184,6 +200,29 @@ static int pool_does_not_fit()
     return 0;
 }
 
+// Occupancy is each device's own, asked once, and a failed query is not kept.
+static int occupancy_by_device()
+{
+    static PerDevice known;
+    auto ask = [&](int dev) {
+        g_device = dev;
+        return resident_ctas((void (*)())nullptr, 256, 0, &known);
+    };
+    g_occupancy[0] = 3;
+    g_occupancy[1] = 5;
+    g_occupancy[99] = 7;  // beyond those whose answers are kept
+    EXPECT(ask(0) == 3 && ask(1) == 5 && ask(0) == 3 && ask(1) == 5 && g_occupancy_asked == 2);
+    EXPECT(ask(99) == 7 && ask(99) == 7);
+    EXPECT(ask(2) == 1 && g_last == cudaSuccess);  // fails
+    g_occupancy[2] = 4;
+    EXPECT(ask(2) == 4);
+    g_occupancy[2] = 0;
+    EXPECT(ask(2) == 4);
+    g_device = 0;
+    EXPECT(resident_ctas((void (*)())nullptr, 256, 0) == 3);
+    return 0;
+}
+
 struct Check {
     const char *name;
     int (*fn)();
@@ -193,6 +232,7 @@ static const Check kChecks[] = {
     {"level_ticket_counter", level_ticket_counter},
     {"leaf_item_counter", leaf_item_counter},
     {"pool_does_not_fit", pool_does_not_fit},
+    {"occupancy_by_device", occupancy_by_device},
 };
 
 int main(int argc, char **argv)

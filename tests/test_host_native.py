@@ -19,7 +19,7 @@ def checks(tmp_path_factory):
 
 
 @pytest.mark.parametrize("name", ["queue_leaf_entries", "level_ticket_counter", "leaf_item_counter",
-                                  "pool_does_not_fit"])
+                                  "pool_does_not_fit", "occupancy_by_device"])
 def test_host_rule(checks, name):
     r = subprocess.run([checks, name], stdout=subprocess.PIPE, text=True)
     assert r.returncode == 0, r.stdout
