@@ -48,7 +48,10 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), int grid, int threads, size
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    if (e != cudaSuccess)
+        cudaGetLastError();  // reported here, not by the process's next check
+    return e;
 }
 
 // Answers of resident_ctas, by device (0: not asked yet).

@@ -49,6 +49,15 @@ static cudaError_t fake_occupancy(int *per_sm, K, int, size_t)
     *per_sm = g_occupancy[g_device];
     return *per_sm ? cudaSuccess : (g_last = cudaErrorInvalidDevice);
 }
+static cudaError_t g_launch = cudaSuccess;
+template <typename... A>
+static cudaError_t fake_launch(const cudaLaunchConfig_t *, A...)
+{
+    if (g_launch != cudaSuccess)
+        g_last = g_launch;
+    return g_launch;
+}
+#define cudaLaunchKernelEx fake_launch
 #define cudaGetDevice fake_get_device
 #define cudaOccupancyMaxActiveBlocksPerMultiprocessor fake_occupancy
 #define cudaMalloc fake_malloc
@@ -223,6 +232,18 @@ static int occupancy_by_device()
     return 0;
 }
 
+// A refused launch is reported by its own return value and leaves no error
+// behind; one that went well leaves an error of before alone.
+static int chained_launch_error()
+{
+    g_last = cudaErrorInvalidValue;
+    EXPECT(launch_chained((void (*)())nullptr, 1, 32, 0, nullptr) == cudaSuccess && g_last == cudaErrorInvalidValue);
+    g_launch = cudaErrorLaunchOutOfResources;
+    EXPECT(launch_chained((void (*)())nullptr, 1, 32, 0, nullptr) == cudaErrorLaunchOutOfResources);
+    EXPECT(g_last == cudaSuccess);
+    return 0;
+}
+
 struct Check {
     const char *name;
     int (*fn)();
@@ -233,6 +254,7 @@ static const Check kChecks[] = {
     {"leaf_item_counter", leaf_item_counter},
     {"pool_does_not_fit", pool_does_not_fit},
     {"occupancy_by_device", occupancy_by_device},
+    {"chained_launch_error", chained_launch_error},
 };
 
 int main(int argc, char **argv)

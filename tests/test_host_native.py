@@ -19,7 +19,8 @@ def checks(tmp_path_factory):
 
 
 @pytest.mark.parametrize("name", ["queue_leaf_entries", "level_ticket_counter", "leaf_item_counter",
-                                  "pool_does_not_fit", "occupancy_by_device"])
+                                  "pool_does_not_fit", "occupancy_by_device",
+                                  "chained_launch_error"])
 def test_host_rule(checks, name):
     r = subprocess.run([checks, name], stdout=subprocess.PIPE, text=True)
     assert r.returncode == 0, r.stdout
