@@ -400,7 +400,9 @@ __device__ __forceinline__ uint32_t orbit_step(Orbit &o, uint32_t limit)
         z_update(o.x, o.y, o.cr, o.ci);
         ++o.d;
     }
-    return o.d >= limit ? ORBIT_DONE : ORBIT_RUN;
+    // (the last state is tested here as a block's is: an orbit that it ends
+    // would be taken for one that outlives those of the same dwell)
+    return (o.d >= limit || !z_bounded(o.x, o.y)) ? ORBIT_DONE : ORBIT_RUN;
 }
 
 // Exact dwell of an orbit left pending by orbit_step<K>: its starting state

@@ -303,7 +303,9 @@ __device__ __forceinline__ uint32_t orbit_w_step(OrbitW<A> &o, uint32_t limit)
         A::update(o.x, o.y, o.cr, o.ci);
         ++o.d;
     }
-    return o.d >= limit ? ORBIT_DONE : ORBIT_RUN;
+    // (the last state is tested here as a block's is: an orbit that it ends
+    // would be taken for one that outlives those of the same dwell)
+    return (o.d >= limit || !A::bounded(o.x, o.y)) ? ORBIT_DONE : ORBIT_RUN;
 }
 
 // Exact dwell of a pending orbit: z_d passed, z_{d+K} failed, and failing is
