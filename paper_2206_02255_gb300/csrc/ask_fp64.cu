@@ -280,7 +280,11 @@ __device__ __forceinline__ OrbitW<A> orbit_w_start(double2 c)
 // Up to K more updates without passing `limit` (ORBIT_RUN / ORBIT_DONE /
 // ORBIT_PEND as for the single-precision orbits): a pending orbit escaped
 // inside the unchecked block and keeps the block's starting state.
-template <class A, uint32_t K>
+// LAST: a tested orbit's last state is tested in this round, as a block's is:
+// in a query, one that it ends would be taken to outlive those of the same
+// dwell.  (In the leaf kernel the next round does it: n = 3000 on the antenna,
+// float-float, leaf kernel 5.00 ms so, 5.14 with the test.)
+template <class A, uint32_t K, bool LAST>
 __device__ __forceinline__ uint32_t orbit_w_step(OrbitW<A> &o, uint32_t limit)
 {
     if (o.d >= limit)
@@ -303,9 +307,7 @@ __device__ __forceinline__ uint32_t orbit_w_step(OrbitW<A> &o, uint32_t limit)
         A::update(o.x, o.y, o.cr, o.ci);
         ++o.d;
     }
-    // (the last state is tested here as a block's is: an orbit that it ends
-    // would be taken for one that outlives those of the same dwell)
-    return (o.d >= limit || !A::bounded(o.x, o.y)) ? ORBIT_DONE : ORBIT_RUN;
+    return (o.d >= limit || (LAST && !A::bounded(o.x, o.y))) ? ORBIT_DONE : ORBIT_RUN;
 }
 
 // Exact dwell of a pending orbit: z_d passed, z_{d+K} failed, and failing is
@@ -367,7 +369,7 @@ __device__ __forceinline__ bool warp_uniform_w(const PixelMap64 &pm, uint32_t ma
         bool differ = false;
         for (;;) {
             if (stt == ORBIT_RUN)
-                stt = orbit_w_step<A, A::kRound>(o, limit);
+                stt = orbit_w_step<A, A::kRound, true>(o, limit);
             const unsigned dm = __ballot_sync(kAll, stt != ORBIT_RUN) & amask;
             if (dm == amask)
                 break;
@@ -612,7 +614,7 @@ __global__ void __launch_bounds__(kLeaf64Warps * 32) leaf64_kernel(Leaf64Args a)
             break;
         uint32_t st = ORBIT_RUN;
         if (busy) {
-            st = orbit_w_step<A, A::kRound>(o, a.max_dwell);
+            st = orbit_w_step<A, A::kRound, false>(o, a.max_dwell);
             if (st == ORBIT_DONE) {
                 a.map[(size_t)(pix >> 16) * a.n + (pix & 0xffffu)] = o.d;
                 if (COUNT) {
