@@ -38,6 +38,12 @@ KERNEL_SOURCES = ["paper_2206_02255_gb300/csrc/ask_kernels.cu",
                   "paper_2206_02255_gb300/csrc/ask_internal.h"]
 
 
+def executed(st):
+    """z-updates that a counting render ran: those it counted less those spared
+    by proofs that an orbit stays in the set."""
+    return st["iterations"] - st["spared_iterations"]
+
+
 def recorded_traffic(kernel_key, workload):
     """DRAM bytes per launch of `kernel_key` from the committed ncu record,
     or None if the record is for another workload or the kernels changed
@@ -293,10 +299,11 @@ def measure_large(ctx, dev, local, world, steps=3, warmup=2):
     return {"workload": C["name"], "n": n, "max_dwell": M, "window": list(win),
             "g": g, "r": r, "B": B, "steps": steps, "ms_per_step": ms,
             "gpix_s": world * px / (ms / 1e3) / 1e9, "min_ms": per[0], "max_ms": per[-1],
-            "dwell_iter_s_executed": cst["iterations"] / (ms / 1e3),
+            "dwell_iter_s_executed": executed(cst) / (ms / 1e3),
             "kernels_ms": {"leaf": t["ms_leaf"] / R,
                            "levels": [x / R for x in t["ms_per_level"][:cst["levels"]]]},
-            "leaf_iterations": cst["leaf_iterations"], "levels": cst["levels"],
+            "leaf_iterations": cst["leaf_iterations"],
+            "leaf_iterations_spared": cst["spared_leaf_iterations"], "levels": cst["levels"],
             "leaves": cst["leaves"], "gpu_launches_per_step": cst["kernel_launches"],
             "l2": "output map %.1f GB > 129 MB L2" % (4 * px / 1e9), "clocks": clk}
 
@@ -513,7 +520,12 @@ def run_gpu(args):
     for i, t in enumerate(timing["ms_per_level"]):
         kern["level%d" % i] = t / R
     dom = max(kern, key=kern.get)
-    it_dom = cst["leaf_iterations"] if dom == "leaf" else cst["iterations_per_level"][int(dom[5:])]
+    if dom == "leaf":
+        it_dom, it_spared = cst["leaf_iterations"], cst["spared_leaf_iterations"]
+    else:
+        it_dom = cst["iterations_per_level"][int(dom[5:])]
+        it_spared = cst["spared_iterations_per_level"][int(dom[5:])]
+    it_dom -= it_spared                                   # updates that were run
     achieved = it_dom / (kern[dom] / 1e3) / 1e9           # G dwell-iterations / s
     f_mhz = 2070.0
     try:
@@ -523,8 +535,8 @@ def run_gpu(args):
     # The roofline's unit is the stepwise iteration's 6 FP32-pipe instructions
     # (1 FMUL + 4 FFMA + 1 FADD); "frac_useful_4op" takes the 4 instructions
     # an update costs when the test is amortised over a block (3 FFMA +
-    # 1 FADD), the bound on useful issue.  achieved = the dominant kernel's
-    # dwell iterations (a counting render) / its mean CUDA-event time.
+    # 1 FADD), the bound on useful issue.  achieved = the dwell iterations that
+    # the dominant kernel runs (a counting render) / its mean CUDA-event time.
     peak = sms * 128 * f_mhz * 1e6 / FP32_OPS_PER_ITER / 1e9
     peak4 = sms * 128 * f_mhz * 1e6 / FP32_OPS_PER_UPDATE / 1e9
     key = "leaf_refill_kernel" if dom == "leaf" else "level_kernel_" + dom
@@ -538,9 +550,9 @@ def run_gpu(args):
                 "peak_useful_4op_basis": "%d SMs x 128 FP32 lanes x %.0f MHz / %d FP32-pipe "
                                          "instructions per blocked update (3 FFMA + 1 FADD)"
                                          % (sms, f_mhz, FP32_OPS_PER_UPDATE),
-                "achieved_basis": "%d dwell iterations of the %s kernel (counting render) / "
-                                  "%.4f ms mean CUDA-event time over %d timed steps"
-                                  % (it_dom, dom, kern[dom], R)}
+                "achieved_basis": "%d dwell iterations run by the %s kernel (counting render; %d "
+                                  "more spared by proofs) / %.4f ms mean CUDA-event time over %d "
+                                  "timed steps" % (it_dom, dom, it_spared, kern[dom], R)}
     if clk and clk.get("sm_mhz"):
         roofline["frac_at_sampled_clock"] = achieved / (
             sms * 128 * clk["sm_mhz"] * 1e6 / FP32_OPS_PER_ITER / 1e9)
@@ -652,11 +664,11 @@ def run_gpu(args):
             "config": workload_config(C, g, r, B, blk),
             "method": "ask", "parallelism": "replicas" if world > 1 else "single",
             "tune": swept,
-            "dwell_iter_s": {"executed": cst["iterations"] / (ms_step / 1e3),
+            "dwell_iter_s": {"executed": executed(cst) / (ms_step / 1e3),
                              "exhaustive_equivalent": est["iterations"] / (ms_step / 1e3)},
             "step_ms": step_pct,
             "exhaustive": {"ms": finite(ms_ex), "gpix_s": finite(pixels / (ms_ex / 1e3) / 1e9),
-                           "dwell_iter_s": finite(est["iterations"] / (ms_ex / 1e3)),
+                           "dwell_iter_s": finite(executed(est) / (ms_ex / 1e3)),
                            "block": list(ex_block[0]) if ex_block else None},
             "cdp2": ({"ms_tail_launch": ms_cdp, "ms_fire_and_forget": ms_cdp_fnf,
                       "gpix_s": pixels / (min(ms_cdp, ms_cdp_fnf) / 1e3) / 1e9,
@@ -671,6 +683,9 @@ def run_gpu(args):
             "fills_per_level": cst["fills_per_level"],
             "iterations_per_level": cst["iterations_per_level"],
             "leaf_iterations": cst["leaf_iterations"],
+            "iterations_spared": {"levels": cst["spared_iterations_per_level"],
+                                  "leaf": cst["spared_leaf_iterations"],
+                                  "exhaustive": est["spared_iterations"]},
             "roofline": roofline, "roofline_fill": roofline_fill,
             "cpu_baseline": cpu, "e2e": e2e,
             "gpu_launches": launches_per_step * args.steps,
@@ -788,7 +803,7 @@ def measure_batch(ctx, dev, local, world, rank, nframes, steps, warmup, probes=6
            "speedup_batch_vs_per_frame": ms_frame / ms_batch,
            "speedup_persistent_vs_chain": ms_batch / ms_pers,
            "speedup_persistent_vs_per_frame": ms_frame / ms_pers,
-           "dwell_iter_s": {"executed": st["iterations"] / (ms_batch / 1e3)},
+           "dwell_iter_s": {"executed": executed(st) / (ms_batch / 1e3)},
            "tuned_probes": tuner.summary(), "clocks": clk, "steps": steps}
     if full:
         res["model_vs_measured"] = probe_models
@@ -1088,7 +1103,7 @@ def run_deep(args):
             "exhaustive64": {"ms": ms_ex, "gpix_s": gp(ms_ex),
                              "fp64_gops": ex_gops, "frac_of_nominal_fp64": ex_gops / FP64_PEAK_GOPS},
             "speedup_vs_exhaustive": ms_ex / ms_ask,
-            "dwell_iter_s": {"executed": cst["iterations"] / (ms_ask / 1e3),
+            "dwell_iter_s": {"executed": executed(cst) / (ms_ask / 1e3),
                              "exhaustive_equivalent": ex_iters / (ms_ask / 1e3)},
             "mismatch_vs_exhaustive_pixels": mism,
             "levels": cst["levels"], "leaves": cst["leaves"],

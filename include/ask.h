@@ -165,10 +165,12 @@ typedef struct {
     uint64_t fill_pixels;                      /* ASK_FLAG_COUNT only */
     uint64_t leaf_pixels;                      /* ASK_FLAG_COUNT only */
     uint64_t border_pixels;                    /* ASK_FLAG_COUNT only */
-    uint64_t iterations;                       /* ASK_FLAG_COUNT only: z-updates counted (an orbit
-                                                * found to repeat itself counts max_dwell) */
-    uint64_t iterations_per_level[ASK_MAX_LEVELS]; /* ASK_FLAG_COUNT, ASK: z-updates of level i */
-    uint64_t leaf_iterations;                  /* ASK_FLAG_COUNT, ASK: z-updates of the leaf kernel */
+    uint64_t iterations;                       /* ASK_FLAG_COUNT only: z-updates, an orbit proven
+                                                * to stay in the set (a repeated state, or one
+                                                * that cannot leave a disc) counted as max_dwell;
+                                                * ask_spared_read: those of them not run */
+    uint64_t iterations_per_level[ASK_MAX_LEVELS]; /* ASK_FLAG_COUNT, ASK: those of level i */
+    uint64_t leaf_iterations;                  /* ASK_FLAG_COUNT, ASK: those of the leaf kernel */
     float ms_total;                            /* device time of the render */
     float ms_per_level[ASK_MAX_LEVELS];        /* ASK: device time of level kernel i */
     float ms_leaf;                             /* ASK: leaf kernel (by default with the
@@ -195,6 +197,14 @@ typedef struct {
     float ms_leaf;                             /* ASK: leaf kernel (as in ask_stats) */
     float ms_fill;                             /* ASK: deferred-fill kernel (as in ask_stats) */
 } ask_timing;
+
+/* Of the z-updates that a render with ASK_FLAG_COUNT counts, those that were
+ * not run: of orbits proven to stay, from the proof to max_dwell. */
+typedef struct {
+    uint64_t iterations;                           /* of ask_stats.iterations */
+    uint64_t iterations_per_level[ASK_MAX_LEVELS]; /* of iterations_per_level */
+    uint64_t leaf_iterations;                      /* of leaf_iterations */
+} ask_spared;
 
 typedef struct ask_ctx ask_ctx;
 
@@ -274,6 +284,10 @@ void ask_graph_destroy(ask_graph *graph);
  * with ASK_FLAG_TIMING since the previous call into *out and forget them.
  * The renders must all have been issued on `stream` (or be complete). */
 ask_status ask_timing_read(ask_ctx *ctx, void *stream, ask_timing *out);
+
+/* The updates spared by the render whose counters were read last (a call with
+ * stats, or ask_check); all 0 if it did not count.  Host only. */
+ask_status ask_spared_read(const ask_ctx *ctx, ask_spared *out);
 
 /* Synchronise `stream` and return (and clear) any latched device error. */
 ask_status ask_check(ask_ctx *ctx, void *stream);

@@ -84,6 +84,17 @@ class Stats(ctypes.Structure):
         }
 
 
+class Spared(ctypes.Structure):
+    _fields_ = [("iterations", ctypes.c_uint64),
+                ("iterations_per_level", ctypes.c_uint64 * ASK_MAX_LEVELS),
+                ("leaf_iterations", ctypes.c_uint64)]
+
+    def as_dict(self, levels):
+        return {"spared_iterations": self.iterations,
+                "spared_iterations_per_level": list(self.iterations_per_level[:levels]),
+                "spared_leaf_iterations": self.leaf_iterations}
+
+
 class Timing(ctypes.Structure):
     _fields_ = [("renders", ctypes.c_uint32), ("dropped", ctypes.c_uint32),
                 ("levels", ctypes.c_uint32), ("method", ctypes.c_uint32),
@@ -130,6 +141,7 @@ SIGNATURES = {
                                        ctypes.c_void_p, _P(Stats)]),
     "ask_check": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
     "ask_timing_read": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, _P(Timing)]),
+    "ask_spared_read": (ctypes.c_int, [ctypes.c_void_p, _P(Spared)]),
     "ask_plan_levels": (ctypes.c_int, [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_uint32,
                                        ctypes.c_uint32, _P(ctypes.c_uint32), _P(ctypes.c_uint64),
                                        ctypes.c_uint32, _P(ctypes.c_uint32)]),
@@ -307,6 +319,15 @@ class Context:
         msg = lib().ask_last_error(self._h)
         raise AskError(st, "%s: %s (%s)" % (what, status_str(st), (msg or b"").decode()))
 
+    def _stats(self, st_obj):
+        """The stats dict of a call, with the counted updates that its proofs
+        spared (``ask_spared_read``)."""
+        sp = Spared()
+        st = lib().ask_spared_read(self._h, ctypes.byref(sp))
+        if st != OK:
+            self._raise(st, "ask_spared_read")
+        return dict(st_obj.as_dict(), **sp.as_dict(st_obj.levels))
+
     def reserve(self, method, n, params=None):
         st = lib().ask_reserve(self._h, _method(method), n,
                                ctypes.byref(params) if params is not None else None)
@@ -334,7 +355,7 @@ class Context:
                               ctypes.byref(st_obj) if st_obj is not None else None)
         if st != OK:
             self._raise(st, "ask_render")
-        return (out, st_obj.as_dict()) if stats else out
+        return (out, self._stats(st_obj)) if stats else out
 
     def render64(self, method, window, n, max_dwell, params=None, out=None, stream=None,
                  stats=False):
@@ -355,7 +376,7 @@ class Context:
                                 ctypes.byref(st_obj) if st_obj is not None else None)
         if st != OK:
             self._raise(st, "ask_render64")
-        return (out, st_obj.as_dict()) if stats else out
+        return (out, self._stats(st_obj)) if stats else out
 
     def render_host(self, method, window, n, max_dwell, params=None, out=None, stream=None,
                     stats=False):
@@ -383,7 +404,7 @@ class Context:
                                    ctypes.byref(st_obj) if st_obj is not None else None)
         if st != OK:
             self._raise(st, "ask_render_host")
-        return (out, st_obj.as_dict()) if stats else out
+        return (out, self._stats(st_obj)) if stats else out
 
     def timing_read(self, stream=None):
         """Per-kernel device times summed over the ASK_FLAG_TIMING renders
@@ -433,7 +454,7 @@ class Context:
                                         ctypes.byref(st_obj) if st_obj is not None else None)
             if st != OK:
                 self._raise(st, "ask_render_batch")
-            out = st_obj.as_dict() if stats else None
+            out = self._stats(st_obj) if stats else None
         for f in deep:
             self.render64("ask", f["window"], int(f["n"]), int(f["max_dwell"]),
                           make_params(int(f["g"]), int(f["r"]), int(f["B"])), out=f["out"],
@@ -441,7 +462,7 @@ class Context:
         if stats:
             if out is None:
                 s.synchronize()
-                out = Stats().as_dict()
+                out = dict(Stats().as_dict(), **Spared().as_dict(0))
             out["fp64_frames"] = len(deep)
         return out
 

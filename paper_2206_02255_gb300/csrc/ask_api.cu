@@ -92,6 +92,7 @@ struct ask_ctx {
     uint64_t ring_head = 0, ring_tail = 0;
     uint32_t ring_dropped = 0;
     size_t cdp_pending = 0;
+    ask_spared spared = {};              // of the render whose counters were read last
     char err[256];
 };
 
@@ -384,6 +385,9 @@ ask_status read_counters(ask_ctx *ctx, cudaStream_t s)
         e = cudaStreamSynchronize(s);
     if (e != cudaSuccess)
         return cuda_err(ctx, e, "reading device counters");
+    ctx->spared.iterations = ctx->h_ctr->spared;
+    std::memcpy(ctx->spared.iterations_per_level, ctx->h_ctr->level_spared, sizeof(ctx->h_ctr->level_spared));
+    ctx->spared.leaf_iterations = ctx->h_ctr->leaf_spared;
     const uint32_t err = ctx->h_ctr->error;
     if (err) {
         e = cudaMemsetAsync(&ctx->ctr->error, 0, sizeof(uint32_t), s);
@@ -1393,6 +1397,14 @@ ask_status ask_timing_read(ask_ctx *ctx, void *stream, ask_timing *out)
     }
     ctx->ring_tail = ctx->ring_head;
     ctx->ring_dropped = 0;
+    return ASK_OK;
+}
+
+ask_status ask_spared_read(const ask_ctx *ctx, ask_spared *out)
+{
+    if (!ctx || !out)
+        return ASK_EINVAL;
+    *out = ctx->spared;
     return ASK_OK;
 }
 

@@ -93,7 +93,7 @@ __device__ __forceinline__ void cdp2_region(const CdpArgs &a, const Region &g, u
     const uint32_t stage_cap = min(4u * side, kStageMax);
     const uint32_t sc = ceil_div_u32(side, a.r);
     const bool split = side > 1u && sc >= a.B;
-    unsigned long long it = 0;
+    Updates it;
     const uint32_t P = perimeter_size(g.w, g.h);
     uint32_t dmin, dmax;
 
@@ -228,7 +228,7 @@ __device__ __forceinline__ void cdp2_region(const CdpArgs &a, const Region &g, u
                         const uint32_t px = g.x0 + tx0 + threadIdx.x, py = g.y0 + ty0 + threadIdx.y;
                         if (px < g.x0 + g.w && py < g.y0 + g.h && !on_perimeter(g, px, py)) {
                             const float2 c = pixel_c(a.pm, px, py);
-                            const uint32_t d = dwell(c.x, c.y, a.max_dwell);
+                            const uint32_t d = dwell(c.x, c.y, a.max_dwell, &it.spared);
                             a.map[(size_t)py * a.n + px] = d;
                             it += d;
                         }
@@ -239,11 +239,8 @@ __device__ __forceinline__ void cdp2_region(const CdpArgs &a, const Region &g, u
             }
         }
     }
-    if (a.count) {
-        it = warp_sum_u64(it);
-        if (lane == 0 && it)
-            atomicAdd(&a.ctr->iterations, it);
-    }
+    if (a.count)
+        count_updates(a.ctr, nullptr, nullptr, it, lane);
 }
 
 __global__ void __launch_bounds__(1024) cdp2_list_kernel(CdpArgs a, uint32_t side, uint32_t level);

@@ -10,6 +10,38 @@
 
 namespace ask {
 
+// z-updates of a counting render.  counted: as far as each orbit was followed,
+// an orbit proven to stay with max_dwell; spared: those of them that were not
+// run, from the proof to max_dwell.
+struct Updates {
+    unsigned long long counted = 0, spared = 0;
+    __device__ __forceinline__ void operator+=(uint32_t d) { counted += d; }
+};
+
+// Add a whole warp's updates to the render's counters and to those of a part
+// of it (NULL: none).
+__device__ __forceinline__ void count_updates(DevCounters *ctr, unsigned long long *part,
+                                              unsigned long long *part_spared, Updates it, uint32_t lane)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        it.counted += __shfl_xor_sync(0xffffffffu, it.counted, o);
+        it.spared += __shfl_xor_sync(0xffffffffu, it.spared, o);
+    }
+    if (lane != 0)
+        return;
+    if (it.counted) {
+        atomicAdd(&ctr->iterations, it.counted);
+        if (part)
+            atomicAdd(part, it.counted);
+    }
+    if (it.spared) {
+        atomicAdd(&ctr->spared, it.spared);
+        if (part)
+            atomicAdd(part_spared, it.spared);
+    }
+}
+
 // Updates per unchecked block of the dwell loops: the first and the others of
 // the loop with proofs, and those of the plain loop (see dwell()).
 constexpr int kFirstBlock = 16;
@@ -249,8 +281,10 @@ __device__ __forceinline__ uint32_t dwell_in_block(float x, float y, float cr, f
 // boundary, where proofs come late or never (n = 16384, cap 2048: ASK-MBR 3.80
 // ms with proofs, 3.58 without; tiled leaves 2.55 -> 2.41; DP-MBR 5.87 -> 5.60).
 // CDP2's own leaves keep them: n = 1024, B = 32 0.410 ms without, 0.296 with.
+// `spared` (or NULL) gains the updates that a proof saved.
 template <bool PROVE = true>
-__device__ __forceinline__ uint32_t dwell(float cr, float ci, uint32_t max_dwell)
+__device__ __forceinline__ uint32_t dwell(float cr, float ci, uint32_t max_dwell,
+                                          unsigned long long *spared = nullptr)
 {
     float x = 0.0f, y = 0.0f;
     uint32_t d = 0;
@@ -294,8 +328,11 @@ __device__ __forceinline__ uint32_t dwell(float cr, float ci, uint32_t max_dwell
                         break;
                 }
             }
-            if (in)
+            if (in) {
+                if (spared)
+                    *spared += max_dwell - d;
                 return max_dwell;
+            }
             if (esc)
                 return dwell_in_block<kUnroll>(x, y, cr, ci, d);
         } else {
@@ -665,13 +702,14 @@ __device__ __forceinline__ bool resolve_block(const float *x0, const float *y0, 
 // took to enter it.  w: the region's common dwell as far as known (kNone32:
 // none yet); orbits stop at w + 1.  ps (or NULL): the region's shared state
 // {common dwell, differs}, read along the way, `lag` rounds between a load and
-// its use.  On GROUP_SAME d holds the dwells (above w: anything above w).
+// its use.  On GROUP_SAME d holds the dwells (above w: anything above w).  `it`
+// gains the updates that proofs spared.
 template <uint32_t K, int NS, bool PROVE>
 __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max_dwell,
                                                 const uint32_t *px, const uint32_t *py,
                                                 const bool *active, uint32_t rnd, uint32_t w,
                                                 const volatile uint32_t *ps, uint32_t lag,
-                                                uint32_t lane, uint32_t *d)
+                                                uint32_t lane, uint32_t *d, Updates &it)
 {
     float x[NS], y[NS], cr[NS], ci[NS];
     float bx[NS], by[NS], ax[NS], ay[NS], r2[NS];
@@ -786,6 +824,8 @@ __device__ __forceinline__ uint32_t query_group(const PixelMap &pm, uint32_t max
                                           (x[i] == bx[i] && y[i] == by[i]));
             if (run[i] && ok)
                 d[i] = in ? max_dwell : n;
+            if (run[i] && ok && in)
+                it.spared += max_dwell - n;
             // (at the limit an orbit has ended: its dwell may equal that of
             // one whose last state escaped)
             run[i] = run[i] && ok && !in && n < limit;
@@ -846,7 +886,7 @@ __device__ __forceinline__ uint32_t spread_group(const PixelMap &pm, uint32_t ma
                                                  uint32_t first, uint32_t stride, uint32_t base,
                                                  uint32_t P, uint32_t rnd, uint32_t w,
                                                  const volatile uint32_t *ps, uint32_t lag, uint32_t lane,
-                                                 uint32_t &vmin, uint32_t &vmax, unsigned long long &it)
+                                                 uint32_t &vmin, uint32_t &vmax, Updates &it)
 {
     uint32_t px[NS], py[NS], d[NS];
     bool active[NS];
@@ -859,7 +899,7 @@ __device__ __forceinline__ uint32_t spread_group(const PixelMap &pm, uint32_t ma
         if (active[i])
             perimeter_pixel(g, k, px[i], py[i]);
     }
-    const uint32_t r = query_group<K, NS, PROVE>(pm, max_dwell, px, py, active, rnd, w, ps, lag, lane, d);
+    const uint32_t r = query_group<K, NS, PROVE>(pm, max_dwell, px, py, active, rnd, w, ps, lag, lane, d, it);
 #pragma unroll
     for (int i = 0; i < NS; ++i)
         if (active[i])
@@ -875,7 +915,7 @@ __device__ __forceinline__ uint32_t spread_group(const PixelMap &pm, uint32_t ma
 template <uint32_t K, int NS, bool PROVE>
 __device__ __forceinline__ bool warp_perimeter_uniform(const PixelMap &pm, uint32_t max_dwell,
                                                        const Region &g, uint32_t lane, uint32_t rnd,
-                                                       uint32_t *w_out, unsigned long long &it)
+                                                       uint32_t *w_out, Updates &it)
 {
     const uint32_t P = perimeter_size(g.w, g.h);
     const uint32_t groups = (P + 32u * NS - 1u) / (32u * NS);
@@ -898,7 +938,7 @@ __device__ __forceinline__ bool warp_perimeter_uniform(const PixelMap &pm, uint3
 __device__ __forceinline__ bool cta_perimeter_uniform(const PixelMap &pm, uint32_t max_dwell,
                                                       const Region &g, uint32_t tid, uint32_t T,
                                                       uint32_t *s_flag, uint32_t *s_w,
-                                                      uint32_t *w_out, unsigned long long &it)
+                                                      uint32_t *w_out, Updates &it)
 {
     const uint32_t P = perimeter_size(g.w, g.h);
     const uint32_t lane = tid & 31u;

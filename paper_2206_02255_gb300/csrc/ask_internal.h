@@ -24,11 +24,13 @@ struct DevCounters {
                                             // where the producer does not order its leaves)
     uint32_t error;                         // ERR_* bits, latched
     unsigned long long iterations;          // COUNT mode: z-updates
+    unsigned long long spared;              // COUNT mode: those of them not run (proofs of staying)
     unsigned long long fill_pixels;         // COUNT mode
     unsigned long long leaf_pixels;         // COUNT mode
     unsigned long long border_pixels;       // COUNT mode
     unsigned long long level_iters[ASK_MAX_LEVELS];  // COUNT mode: z-updates of level i
     unsigned long long leaf_iters;          // COUNT mode: z-updates of the leaf kernel
+    unsigned long long level_spared[ASK_MAX_LEVELS], leaf_spared;  // COUNT mode: of these, not run
     unsigned long long deferred_fill_pixels; // COUNT mode: pixels of the deferred-fill list
     uint32_t work[ASK_MAX_LEVELS];          // next work item a level kernel hands out
     uint32_t leaf_work;                     // next leaf the leaf kernel hands out

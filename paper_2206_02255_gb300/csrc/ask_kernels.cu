@@ -69,17 +69,15 @@ __global__ void __launch_bounds__(1024) exhaustive_kernel(uint32_t *__restrict__
     const uint32_t ty = tile / tiles_x, tx = tile - ty * tiles_x;
     const uint32_t px = tx * blockDim.x + threadIdx.x;
     const uint32_t py = ty * blockDim.y + threadIdx.y;
-    uint32_t d = 0;
+    Updates it;
     if (px < n && py < n) {
         const float2 c = pixel_c(pm, px, py);
-        d = dwell(c.x, c.y, max_dwell);
+        const uint32_t d = dwell(c.x, c.y, max_dwell, COUNT ? &it.spared : nullptr);
         map[(size_t)py * n + px] = d;
+        it += d;
     }
-    if (COUNT) {
-        const unsigned long long s = warp_sum_u64(d);
-        if ((threadIdx.x + threadIdx.y * blockDim.x) % 32u == 0u && s)
-            atomicAdd(&ctr->iterations, s);
-    }
+    if (COUNT)
+        count_updates(ctr, nullptr, nullptr, it, (threadIdx.x + threadIdx.y * blockDim.x) % 32u);
 }
 
 // Order probe of a region (the order in which the region tables and the
@@ -316,14 +314,14 @@ __device__ __forceinline__ void flush_batch(const LevelArgs &a, WarpBatch<BATCH>
 // every dwell is computed and written; st.x / st.y collect min / max.
 __device__ __forceinline__ void chunk_exact(const FView &a, const Region &g, uint32_t k0,
                                             uint32_t k1, uint4 *st, uint32_t lane,
-                                            unsigned long long &it)
+                                            Updates &it)
 {
     uint32_t dmin = kNone, dmax = 0u;
     for (uint32_t k = k0 + lane; k < k1; k += 32u) {
         uint32_t px, py;
         perimeter_pixel(g, k, px, py);
         const float2 c = pixel_c(a.pm, px, py);
-        const uint32_t d = dwell(c.x, c.y, a.max_dwell);
+        const uint32_t d = dwell(c.x, c.y, a.max_dwell, &it.spared);
         a.map[(size_t)py * a.n + px] = d;
         dmin = min(dmin, d);
         dmax = max(dmax, d);
@@ -338,18 +336,14 @@ __device__ __forceinline__ void chunk_exact(const FView &a, const Region &g, uin
 }
 
 // A warp's counts of a level (COUNT mode).
-__device__ __forceinline__ void count_level(const LevelArgs &a, unsigned long long it, unsigned long long bpx,
-                                            unsigned long long fpx, unsigned long long dpx, uint32_t lane)
+__device__ __forceinline__ void count_level(const LevelArgs &a, Updates it, unsigned long long bpx, unsigned long long fpx,
+                                            unsigned long long dpx, uint32_t lane)
 {
-    it = warp_sum_u64(it);
+    count_updates(a.ctr, &a.ctr->level_iters[a.level], &a.ctr->level_spared[a.level], it, lane);
     bpx = warp_sum_u64(bpx);
     fpx = warp_sum_u64(fpx);
     dpx = warp_sum_u64(dpx);
     if (lane == 0) {
-        if (it) {
-            atomicAdd(&a.ctr->iterations, it);
-            atomicAdd(&a.ctr->level_iters[a.level], it);
-        }
         if (bpx)
             atomicAdd(&a.ctr->border_pixels, bpx);
         if (fpx)
@@ -426,7 +420,8 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
     b.dwell = 0;
     b.sc = b.r = 1u;
     uint32_t j = 0;
-    unsigned long long it = 0, bpx = 0, fpx = 0, dpx = 0;
+    Updates it;
+    unsigned long long bpx = 0, fpx = 0, dpx = 0;
 
     // The regions from the front of the table come first and are handed out one
     // item at a time: their costs differ by orders of magnitude (a uniform
@@ -508,7 +503,7 @@ __global__ void __launch_bounds__(256, NS == 1 ? kLevelMinBlocks1 : kLevelMinBlo
                     uint32_t px, py;
                     perimeter_pixel(g, k, px, py);
                     const float2 c = pixel_c(f.pm, px, py);
-                    const uint32_t d = dwell(c.x, c.y, f.max_dwell);
+                    const uint32_t d = dwell(c.x, c.y, f.max_dwell, COUNT ? &it.spared : nullptr);
                     dmin = min(dmin, d);
                     dmax = max(dmax, d);
                     if (k < kWarpStage)
@@ -619,7 +614,8 @@ __global__ void __launch_bounds__(256, kLevelMinBlocks2) level_cta_kernel(LevelA
     if (blockIdx.x == 0 && threadIdx.x == 0 &&
         (unsigned long long)a.ctr->count[a.level] + a.ctr->back[a.level] > a.in_cap)
         atomicOr(&a.ctr->error, ERR_OLT_OVERFLOW);
-    unsigned long long it = 0, bpx = 0, fpx = 0, dpx = 0;
+    Updates it;
+    unsigned long long bpx = 0, fpx = 0, dpx = 0;
     for (uint32_t li = blockIdx.x; li < count; li += gridDim.x) {
         const T e = static_cast<const T *>(a.olt_in)[table_slot(li, front, a.in_cap)];
         const Region g = R::region(e);
@@ -698,7 +694,8 @@ __global__ void __launch_bounds__(1024) leaf_kernel(LeafArgs a, uint32_t leaf_ca
     uint32_t front, nleaves;
     leaf_extent(a.ctr, leaf_cap, front, nleaves);
     const unsigned long long total = (unsigned long long)nleaves * tiles_per_leaf;
-    unsigned long long it = 0, lpx = 0;
+    Updates it;
+    unsigned long long lpx = 0;
     for (unsigned long long item = blockIdx.x; item < total; item += gridDim.x) {
         const uint32_t leaf = (uint32_t)(item / tiles_per_leaf);
         const uint32_t t = (uint32_t)(item - (unsigned long long)leaf * tiles_per_leaf);
@@ -717,16 +714,11 @@ __global__ void __launch_bounds__(1024) leaf_kernel(LeafArgs a, uint32_t leaf_ca
         }
     }
     if (COUNT) {
-        it = warp_sum_u64(it);
+        const uint32_t lane = (threadIdx.x + threadIdx.y * blockDim.x) % 32u;
+        count_updates(a.ctr, &a.ctr->leaf_iters, &a.ctr->leaf_spared, it, lane);
         lpx = warp_sum_u64(lpx);
-        if ((threadIdx.x + threadIdx.y * blockDim.x) % 32u == 0u) {
-            if (it) {
-                atomicAdd(&a.ctr->iterations, it);
-                atomicAdd(&a.ctr->leaf_iters, it);
-            }
-            if (lpx)
-                atomicAdd(&a.ctr->leaf_pixels, lpx);
-        }
+        if (lane == 0u && lpx)
+            atomicAdd(&a.ctr->leaf_pixels, lpx);
     }
 }
 
@@ -810,7 +802,8 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocks) leaf_refi
     src.extent = &extent;
     uint32_t srcst = SRC_MORE;
     cursor_reset(w.cursor, lane);
-    unsigned long long it = 0, lpx = 0;
+    Updates it;
+    unsigned long long lpx = 0;
     PrePassFeed<COUNT, BATCH, LeafList<BATCH>> feed{src};
     // a small batch: pre-passes only, the survivors to the pool while it has room
     if (BATCH && a.pool != nullptr)
@@ -858,7 +851,8 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kRefillMinBlocks) pool_kern
     feed.total = total;
     feed.next = kPoolTake * (blockIdx.x + gridDim.x * rank);
     feed.first_end = kPoolTake * gridDim.x * per_cta;
-    unsigned long long it = 0, lpx = 0;
+    Updates it;
+    unsigned long long lpx = 0;
     run_orbits<COUNT, true>(a, feed, SRC_MORE, w, f, lane, it, lpx);
     finish_orbits<COUNT, true>(a, w, f, lane, it, lpx);
 }

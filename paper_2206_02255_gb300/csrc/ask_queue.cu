@@ -231,7 +231,7 @@ __device__ __forceinline__ void process_item(const QueueArgs &q, uint32_t t, uin
     const FView f = view_frame(q.frames, frame, level);
     const uint32_t C = fd.chunks[level];
     const uint32_t P = perimeter_size(g.w, g.h);
-    unsigned long long it = 0;
+    Updates it;
     bool decided = false, uniform = false;
     uint32_t wv = 0;
     if (C <= 1u) {
@@ -241,13 +241,8 @@ __device__ __forceinline__ void process_item(const QueueArgs &q, uint32_t t, uin
         uint4 *st = q.rst + aux;
         decided = chunk_decides(chunk_query<1>(f, g, P, c, C, st, 1u, lane, it), st, C, lane, uniform, wv);
     }
-    if (COUNT) {
-        it = warp_sum_u64(it);
-        if (lane == 0 && it) {
-            atomicAdd(&q.ctr->iterations, it);
-            atomicAdd(&q.ctr->level_iters[level], it);
-        }
-    }
+    if (COUNT)
+        count_updates(q.ctr, &q.ctr->level_iters[level], &q.ctr->level_spared[level], it, lane);
     if (!decided) {
         finish_item(q, epoch, lane);
         return;
@@ -414,7 +409,8 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kQueueMinBlocks) queue_kern
     Slot s[2];
     slot_reset(s[0]);
     slot_reset(s[1]);
-    unsigned long long it = 0, lpx = 0;
+    Updates it;
+    unsigned long long lpx = 0;
 
     uint32_t rt = kNone;      // region ticket held
     bool rclosed = false;     // no region item will come any more
@@ -506,16 +502,10 @@ __global__ void __launch_bounds__(kRefillWarps * 32, kQueueMinBlocks) queue_kern
             ++lpx;
     }
     if (COUNT) {
-        it = warp_sum_u64(it);
+        count_updates(a.ctr, &a.ctr->leaf_iters, &a.ctr->leaf_spared, it, lane);
         lpx = warp_sum_u64(lpx);
-        if (lane == 0) {
-            if (it) {
-                atomicAdd(&a.ctr->iterations, it);
-                atomicAdd(&a.ctr->leaf_iters, it);
-            }
-            if (lpx)
-                atomicAdd(&a.ctr->leaf_pixels, lpx);
-        }
+        if (lane == 0 && lpx)
+            atomicAdd(&a.ctr->leaf_pixels, lpx);
     }
     // the last warp to leave stores the epoch, so the next render's items
     // are told apart from this render's

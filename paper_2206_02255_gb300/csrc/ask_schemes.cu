@@ -49,7 +49,8 @@ __global__ void __launch_bounds__(1024) region_level_kernel(LevelArgs a)
     uint2 *leaves = static_cast<uint2 *>(a.leaves);
     DevCounters *ctr = a.ctr;
     const uint32_t count = min(ctr->count[a.level], a.olt_cap);
-    unsigned long long it = 0, bpx = 0, fpx = 0;
+    Updates it;
+    unsigned long long bpx = 0, fpx = 0;
 
     for (;;) {
         if (tid == 0) {
@@ -116,11 +117,7 @@ __global__ void __launch_bounds__(1024) region_level_kernel(LevelArgs a)
         __syncthreads();  // s_* are rewritten by the next item
     }
     if (COUNT) {
-        it = warp_sum_u64(it);
-        if (lane == 0 && it) {
-            atomicAdd(&ctr->iterations, it);
-            atomicAdd(&ctr->level_iters[a.level], it);
-        }
+        count_updates(ctr, &ctr->level_iters[a.level], &ctr->level_spared[a.level], it, lane);
         if (tid == 0) {
             if (bpx)
                 atomicAdd(&ctr->border_pixels, bpx);
@@ -139,7 +136,8 @@ __global__ void __launch_bounds__(1024) region_leaf_kernel(LeafArgs a)
     const uint32_t tid = threadIdx.x + threadIdx.y * blockDim.x;
     const uint2 *leaves = static_cast<const uint2 *>(a.leaves);
     const uint32_t nleaves = min(a.ctr->leaf_count, a.leaf_cap);
-    unsigned long long it = 0, lpx = 0;
+    Updates it;
+    unsigned long long lpx = 0;
     for (;;) {
         if (tid == 0)
             s_item = atomicAdd(&a.ctr->leaf_work, 1u);
@@ -165,16 +163,10 @@ __global__ void __launch_bounds__(1024) region_leaf_kernel(LeafArgs a)
         }
     }
     if (COUNT) {
-        it = warp_sum_u64(it);
+        count_updates(a.ctr, &a.ctr->leaf_iters, &a.ctr->leaf_spared, it, tid & 31u);
         lpx = warp_sum_u64(lpx);
-        if ((tid & 31u) == 0u) {
-            if (it) {
-                atomicAdd(&a.ctr->iterations, it);
-                atomicAdd(&a.ctr->leaf_iters, it);
-            }
-            if (lpx)
-                atomicAdd(&a.ctr->leaf_pixels, lpx);
-        }
+        if ((tid & 31u) == 0u && lpx)
+            atomicAdd(&a.ctr->leaf_pixels, lpx);
     }
 }
 

@@ -101,7 +101,7 @@ constexpr uint32_t kShortRoundsMaxPerimeter = 512;
 template <int NS>
 __device__ __forceinline__ uint32_t chunk_query(const FView &a, const Region &g, uint32_t P, uint32_t c,
                                                 uint32_t chunks, uint4 *st, uint32_t lag,
-                                                uint32_t lane, unsigned long long &it)
+                                                uint32_t lane, Updates &it)
 {
     const volatile uint32_t *ps = reinterpret_cast<const volatile uint32_t *>(st);
     const uint32_t n = P > c ? (P - c + chunks - 1u) / chunks : 0u;
@@ -226,7 +226,7 @@ __device__ __forceinline__ void store_dwell(const LeafArgs &a, uint32_t frame, u
 // z = 0) take the tested loop instead.  u = (count, py << 16 | px).
 template <bool COUNT, bool BATCH>
 __device__ __forceinline__ void finish_parked(const LeafArgs &a, float4 s, uint2 u, uint32_t frame,
-                                              unsigned long long &it)
+                                              Updates &it)
 {
     const LView v = leaf_view<BATCH>(a, frame);
     const uint32_t px = u.y & 0xffffu, py = u.y >> 16;
@@ -507,7 +507,7 @@ __device__ __forceinline__ void push_survivor(WarpLeaf<BATCH> &w, const WarpFill
 template <bool COUNT, bool BATCH, typename Src>
 __device__ __forceinline__ uint32_t pre_pass(const LeafArgs &a, Src &src, uint32_t &srcst,
                                              WarpLeaf<BATCH> &w, WarpFill &f, uint32_t lane,
-                                             unsigned long long &it, unsigned long long &lpx)
+                                             Updates &it, unsigned long long &lpx)
 {
     uint32_t pix0 = 0, pix1 = 0, fr0 = 0, fr1 = 0;
     uint32_t base = 0;
@@ -719,7 +719,7 @@ __device__ __forceinline__ void fold_slot1(WarpLeaf<BATCH> &w, WarpFill &f, Slot
 // (running the block again changes nothing).  Returns whether it waits.
 template <bool COUNT, bool BATCH>
 __device__ __forceinline__ bool settle_slot(const LeafArgs &a, Slot &s, float x, float y,
-                                            unsigned long long &it, unsigned long long &lpx)
+                                            Updates &it, unsigned long long &lpx)
 {
     const uint32_t K = 2u * (uint32_t)kLeafUnroll;
     const uint32_t lim = slot_limit<BATCH>(a, s);
@@ -735,6 +735,7 @@ __device__ __forceinline__ bool settle_slot(const LeafArgs &a, Slot &s, float x,
         store_dwell<BATCH>(a, s.frame, s.pix, md);
         if (COUNT) {
             it += md;
+            it.spared += md - s.d;
             ++lpx;
         }
         s.busy = false;
@@ -774,7 +775,7 @@ __device__ __forceinline__ void half_block(float *x, float *y, const float *cr, 
 template <bool COUNT, bool BATCH, int NS>
 __device__ __forceinline__ bool refill_round(const LeafArgs &a, WarpLeaf<BATCH> &w, WarpFill &f,
                                              Slot *s, uint32_t thr, uint32_t lane,
-                                             unsigned long long &it, unsigned long long &lpx)
+                                             Updates &it, unsigned long long &lpx)
 {
     float x[NS], y[NS], cr[NS], ci[NS], mx[NS], my[NS];
 #pragma unroll
@@ -877,7 +878,7 @@ struct PoolFeed {
     uint32_t total, next, first_end;  // entries; the warp's next; where the counter's begin
 
     __device__ __forceinline__ void operator()(const LeafArgs &a, uint32_t &srcst, WarpLeaf<true> &w,
-                                               WarpFill &f, uint32_t lane, unsigned long long &,
+                                               WarpFill &f, uint32_t lane, Updates &,
                                                unsigned long long &)
     {
         if (next == kNone) {
@@ -907,7 +908,7 @@ struct PrePassFeed {
     Src &src;
 
     __device__ __forceinline__ void operator()(const LeafArgs &a, uint32_t &srcst, WarpLeaf<BATCH> &w,
-                                               WarpFill &f, uint32_t lane, unsigned long long &it,
+                                               WarpFill &f, uint32_t lane, Updates &it,
                                                unsigned long long &lpx)
     {
         pre_pass<COUNT, BATCH>(a, src, srcst, w, f, lane, it, lpx);
@@ -919,7 +920,7 @@ struct PrePassFeed {
 template <bool COUNT, bool BATCH, typename Feed>
 __device__ __forceinline__ void run_orbits(const LeafArgs &a, Feed &feed, uint32_t srcst,
                                            WarpLeaf<BATCH> &w, WarpFill &f, uint32_t lane,
-                                           unsigned long long &it, unsigned long long &lpx)
+                                           Updates &it, unsigned long long &lpx)
 {
     Slot s[kSlots];
 #pragma unroll
@@ -953,7 +954,7 @@ __device__ __forceinline__ void run_orbits(const LeafArgs &a, Feed &feed, uint32
 // The orbits still parked after run_orbits, and the warp's counts.
 template <bool COUNT, bool BATCH>
 __device__ __forceinline__ void finish_orbits(const LeafArgs &a, const WarpLeaf<BATCH> &w, const WarpFill &f,
-                                              uint32_t lane, unsigned long long it, unsigned long long lpx)
+                                              uint32_t lane, Updates it, unsigned long long lpx)
 {
     if (lane < f.parked) {
         finish_parked<COUNT, BATCH>(a, w.park_s[lane], w.park_u[lane], BATCH ? w.park_f[lane] : 0u, it);
@@ -961,16 +962,10 @@ __device__ __forceinline__ void finish_orbits(const LeafArgs &a, const WarpLeaf<
             ++lpx;
     }
     if (COUNT) {
-        it = warp_sum_u64(it);
+        count_updates(a.ctr, &a.ctr->leaf_iters, &a.ctr->leaf_spared, it, lane);
         lpx = warp_sum_u64(lpx);
-        if (lane == 0) {
-            if (it) {
-                atomicAdd(&a.ctr->iterations, it);
-                atomicAdd(&a.ctr->leaf_iters, it);
-            }
-            if (lpx)
-                atomicAdd(&a.ctr->leaf_pixels, lpx);
-        }
+        if (lane == 0 && lpx)
+            atomicAdd(&a.ctr->leaf_pixels, lpx);
     }
 }
 
