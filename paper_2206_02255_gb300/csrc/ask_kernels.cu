@@ -945,8 +945,9 @@ static cudaError_t level_launch_sized(const LevelArgs &a, int sms, cudaStream_t 
                               32 * (int)std::min(8u, std::max(1u, (4u * a.side + 63u) / 64u)), 0, s, a);
     if (a.chunks > 1u || (!BATCH && a.side > kLevelSide1))
         return level_launch<COUNT, BATCH, 2, true>(a, sms, s);
-    if (!BATCH && (float)a.side * std::max(a.pm.dx, a.pm.dy) >= kProveExtent)
-        return level_launch<COUNT, BATCH, 1, true>(a, sms, s);
+    if constexpr (!BATCH)
+        if ((float)a.side * std::max(a.pm.dx, a.pm.dy) >= kProveExtent)
+            return level_launch<COUNT, BATCH, 1, true>(a, sms, s);
     return level_launch<COUNT, BATCH, 1, false>(a, sms, s);
 }
 
