@@ -879,8 +879,8 @@ __device__ __forceinline__ void group_range(const bool *active, const uint32_t *
     vmax = __reduce_max_sync(kLaneMask, vmax);
 }
 
-// Group j of the `groups` of 32 * NS pixels that cover the perimeter of g (P
-// pixels), spread over all of it: pixels j, j + groups, j + 2 groups, ...
+// A group of up to 32 * NS of the perimeter pixels of g (P pixels), a stride
+// apart: pixels first + k * stride, k = base, base + 1, ...
 template <uint32_t K, int NS, bool PROVE>
 __device__ __forceinline__ uint32_t spread_group(const PixelMap &pm, uint32_t max_dwell, const Region &g,
                                                  uint32_t first, uint32_t stride, uint32_t base,

@@ -359,7 +359,7 @@ __device__ __forceinline__ void count_level(const LevelArgs &a, Updates it, unsi
 //
 // A level is bound by the latency of its items (each a few trips to L2 and a
 // chain of updates) as much as by its updates, so two orbits a lane (24 warps
-// an SM, 80 registers) are the better half wherever an item has more than 32
+// an SM, up to 80 registers) are the better half wherever an item has more than 32
 // pixels to give: side 18 and up, chunks of 64.  Smaller regions take one orbit
 // a lane and 32 warps.  (Two for the regions of side 16 of n = 16384: 393 us
 // against 371; one up to side 40, n = 1999 without chunks: 316 against 311.)
@@ -383,8 +383,14 @@ constexpr uint32_t kLevelSide1 = 17;
 constexpr unsigned long long kCtaLevelRegions = 2048;
 // Small regions (one orbit a lane) look for orbits that stay only where a
 // region is at least this wide in the plane: nearer to the boundary proofs come
-// too late to pay for the looks (sides of 16 at n = 16384: 374 us with, 366
-// without; at n = 4096: 82 with, 96 without).
+// too late to pay for the looks (level of sides 16 at n = 16384, cap 2048: 374 us
+// with, 366 without; at n = 4096: 82 with, 96 without).  Whole maps without / with,
+// at caps 256, 2048 and 8192: n = 4096 (sides 16, 0.0078 wide) 145 / 146, 361 / 349,
+// 1010 / 883 us; n = 16384 (0.002 wide) 882 / 908, 1651 / 1654, 3830 / 3560.  At
+// caps of many thousand they would pay below this line too.
+// A batch's levels of whole small perimeters, and those of the persistent kernel,
+// do without (64 frames of up to 8192 pixels 38.1 ms, 38.4 with proofs; persistent
+// 45.3 and 45.6; 32 frames of up to 2048 3.18 and 3.10 ms, 3.47 and 3.42).
 constexpr float kProveExtent = 0.004f;
 // A ticket of cheap regions stands for at most kTicketMax of them, as long as
 // every warp gets kTicketsPerWarp tickets (1 at most: 377 us at level 3 of n =

@@ -220,8 +220,9 @@ extern "C" ask_status ask_render_noalloc(const ask_window *window, uint32_t n, u
         a.in_cap = kNoAllocRegions;  // the tables fill from both ends of the whole array
         a.out_cap = kNoAllocRegions;
         a.bound = plan.max_regions[i];
-        // one warp per region and fills in place: no per-region query state
-        // or fill list, so the fixed scratch stays at three tables
+        // a warp per region (a CTA at a level of few regions) and fills in
+        // place: no per-region query state or fill list, so the fixed scratch
+        // stays at three tables
         a.chunks = 1u;
         a.next_chunks = 1u;
         a.rst_in = nullptr;

@@ -51,7 +51,7 @@ namespace {
 enum : uint32_t { QITEM_REGION = 0, QITEM_FILL = 1 };
 
 // Resident CTAs per SM: the region items' latency wants more warps than the
-// leaf work alone (64 registers a thread).
+// leaf work alone (64 registers a thread, 256 bytes of them spilled).
 constexpr int kQueueMinBlocks = 4;
 // Leaf rounds between polls of the held region ticket while a warp is busy.
 constexpr uint32_t kQueuePollRounds = 8;

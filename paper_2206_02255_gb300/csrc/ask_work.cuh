@@ -166,10 +166,14 @@ __device__ __forceinline__ bool chunk_decides(uint32_t r, uint4 *st, uint32_t ch
 // Leaf machinery (see the leaf kernel in ask_kernels.cu)
 // ---------------------------------------------------------------------------
 constexpr int kRefillWarps = 8;    // warps per CTA
-// Resident CTAs per SM.  With two orbits a lane the FP32 pipe is busy enough
-// at 24 warps, and 80 registers leave nothing to spill: at n = 16384 (g=16 r=4
-// B=16) the leaf kernel takes 1.08 ms at 5 CTAs (48 registers, 60 bytes
-// spilled), 0.96 at 4 and 0.93 at 3.
+// Resident CTAs per SM that the registers have to allow: 3 leave 85 a thread, so
+// nothing spills (5 CTAs, 48 registers and 60 bytes spilled took 1.08 ms at n =
+// 16384, g=16 r=4 B=16, against 0.96).  A batch takes 72 and runs 3 CTAs; one
+// frame takes 63 and runs 4.  Held to 3 its leaf kernel alone is faster, 0.933 ms
+// against 0.956, but the chain is slower, probably because the CTAs that start
+// while the level kernel before still holds a part of the SMs stay unevenly
+// spread (n = 16384 1.62 -> 1.89 ms, n = 65536 9.90 -> 11.9, n = 3001 366 -> 397
+// us).
 constexpr int kRefillMinBlocks = 3;
 constexpr int kSlots = 2;          // orbits per lane in the refill loop (four: 0.94-0.99 ms)
 constexpr uint32_t kParkCap = 96;  // parked orbits per warp (fewer than 32 wait, a round adds 64)
