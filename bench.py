@@ -35,6 +35,7 @@ TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "dram_traffic_ask_n16384_d2048.j
 KERNEL_SOURCES = ["paper_2206_02255_gb300/csrc/ask_kernels.cu",
                   "paper_2206_02255_gb300/csrc/ask_work.cuh",
                   "paper_2206_02255_gb300/csrc/ask_device.cuh",
+                  "paper_2206_02255_gb300/csrc/ask_launch.cuh",
                   "paper_2206_02255_gb300/csrc/ask_internal.h"]
 
 
