@@ -335,6 +335,21 @@ __device__ __forceinline__ uint32_t dwell(float cr, float ci, uint32_t max_dwell
             }
             if (esc)
                 return dwell_in_block<kUnroll>(x, y, cr, ci, d);
+            // (less than a block is left: half a block before the tested
+            // updates.  Without, low caps are slower than with no proofs:
+            // CDP2, n = 2048, cap 72, leaves of 64 117 us against 92, 97 so)
+            if (max_dwell - d >= (uint32_t)kFirstBlock) {
+                tx = x;
+                ty = y;
+#pragma unroll
+                for (int k = 0; k < kFirstBlock; ++k)
+                    z_update(tx, ty, cr, ci);
+                if (!z_bounded(tx, ty))
+                    return dwell_in_block<kFirstBlock>(x, y, cr, ci, d);
+                x = tx;
+                y = ty;
+                d += (uint32_t)kFirstBlock;
+            }
         } else {
             while (max_dwell - d >= (uint32_t)kPlainBlock) {
                 const float sx = x, sy = y;
